@@ -10,11 +10,14 @@
 // Pass B (this file) multiplies by the inter-pass twiddle w_n^{i2*k1} as it
 // loads, runs the length-n2 FFTs along the workspace rows and writes element
 // k2 of row k1 to out[k1 + n1*k2]: the transpose that natural output order
-// needs is folded into its store.  The inverse needs no conjugation: it is the
-// forward transform read at index (n - k) mod n, so pass B stores to the
-// reflected position instead.  A CTA takes W adjacent rows (thread t owns row c = t % W,
-// butterfly index tt = t / W), so every output position k2 receives W
+// needs is folded into its store.  A CTA takes W adjacent rows (thread t owns row
+// c = t % W, butterfly index tt = t / W), so every output position k2 receives W
 // consecutive values, W*8 bytes, at once -- whole 32-byte sectors for W >= 4.
+// The inverse is conj(F(conj x)): pass A conjugates as it reads its tile, pass
+// B as it stores.  Reading the forward result at index (n - k) mod n instead
+// needs no conjugation, but its W-value runs end one element off a sector
+// boundary, so every 32-byte store touches two sectors (4 x 2^24 points:
+// 0.854 ms stored reflected, 0.484 conjugated, the forward 0.482).
 // Two HBM passes, 32 bytes per point, as for the 2D transform.
 //
 // The twiddle of a thread's stage-0 operand e (butterfly b = e / R0, leg
@@ -79,7 +82,7 @@ __device__ __forceinline__ float2 root_n(const float2 *__restrict__ lohi, int a)
 template <int N, int E, int W, bool MID>
 __global__ void __launch_bounds__(FsRowShape<N, E, W>::THREADS, FsRowShape<N, E, W>::MINB)
     k_rows_fourstep(const float2 *__restrict__ work, float2 *__restrict__ out, const float2 *__restrict__ tw,
-                    const float2 *__restrict__ lohi, int n1, long long ntiles, int reverse, int *status,
+                    const float2 *__restrict__ lohi, int n1, long long ntiles, int conj_out, int *status,
                     int m_arg) {
     using Sh = FsRowShape<N, E, W>;
     using Eng = typename Sh::Eng;
@@ -95,8 +98,7 @@ __global__ void __launch_bounds__(FsRowShape<N, E, W>::THREADS, FsRowShape<N, E,
     const int t = threadIdx.x;
     const int c = t % W;
     const int tt = t / W;
-    const int mask = reverse ? n1 * m * N - 1 : -1;  // n = n1 * m * N is a power of two
-    const int sgn = reverse ? -1 : 1;
+    const float so = conj_out ? -1.f : 1.f;
     // tile id: transform tr, middle digit k2 (m > 1: three passes), rows
     // k1 = k10 .. k10 + W - 1; workspace row (k1, k2) of transform tr at
     // ((tr * n1 + k1) * m + k2) * N
@@ -155,8 +157,8 @@ __global__ void __launch_bounds__(FsRowShape<N, E, W>::THREADS, FsRowShape<N, E,
                 else v[e] = cmul(x, cmul(base, G[c * Sh::GROW + e]));
             }
         }
-        float2 *dst = out + b * (long long)n1 * m * N;
-        const int off = k10 + n1 * k2m, ostride = n1 * m;
+        float2 *dst = out + b * (long long)n1 * m * N + k10 + n1 * k2m;
+        const int ostride = n1 * m;
         auto after_reads = [&] {
             __syncthreads();
             if (t == 0 && next < ntiles) {
@@ -164,7 +166,10 @@ __global__ void __launch_bounds__(FsRowShape<N, E, W>::THREADS, FsRowShape<N, E,
                 issue(next);
             }
         };
-        auto store = [&](int i, int cc, float2 x) { dst[(sgn * (off + cc + i * ostride)) & mask] = x; };
+        auto store = [&](int i, int cc, float2 x) {
+            x.y *= so;
+            dst[cc + i * ostride] = x;  // < n1 * m * N = n <= 2^26
+        };
         Eng::template run<FftPolicy, true>(v, tile, tw, tt, c, SyncBlock{}, after_reads, store);
     }
 }
@@ -233,7 +238,7 @@ const ColVariant *fourstep_row_variant(int log2n, int e, int w) {
 }
 
 cudaError_t launch_rows_fourstep(const ColVariant &v, const float2 *work, float2 *out, const float2 *tw,
-                                 const float2 *lohi, int n1, int batch, int reverse, int *status, cudaStream_t s,
+                                 const float2 *lohi, int n1, int batch, int conj_out, int *status, cudaStream_t s,
                                  int m) {
     if (v.w < 1 || n1 % v.w || m < 1) return cudaErrorInvalidValue;
     init_fs_rows();
@@ -258,7 +263,7 @@ cudaError_t launch_rows_fourstep(const ColVariant &v, const float2 *work, float2
     long long grid = (long long)sms * (per_sm > 0 ? per_sm : 1);
     if (grid > ntiles) grid = ntiles;
     void *args[] = {(void *)&work,   (void *)&out,     (void *)&tw,     (void *)&lohi, (void *)&n1,
-                    (void *)&ntiles, (void *)&reverse, (void *)&status, (void *)&m};
+                    (void *)&ntiles, (void *)&conj_out, (void *)&status, (void *)&m};
     return cudaLaunchKernel(fn, dim3((unsigned)grid), dim3(v.threads), args, v.smem, s);
 }
 

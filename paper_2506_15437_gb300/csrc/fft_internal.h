@@ -154,11 +154,10 @@ int fourstep_row_e(int n);
 int fourstep_row_w(int n);
 // Pass B: element i2 of row k1 of work [batch][n1][v.n] times w_n^{i2*k1}
 // (from lohi = [w_n^k, k < 8192 | w_n^{8192 k}, k < n/8192]), length-v.n FFTs
-// of the rows, element k2 of row k1 stored at out[b][k] with k = k1 + n1*k2,
-// or at out[b][(n - k) mod n] if reverse (which turns the forward transform
-// into the inverse).
+// of the rows, element k2 of row k1 stored at out[b][k1 + n1*k2], conjugated
+// if conj_out (the inverse; pass A conjugates its inputs).
 cudaError_t launch_rows_fourstep(const ColVariant &v, const float2 *work, float2 *out, const float2 *tw,
-                                 const float2 *lohi, int n1, int batch, int reverse, int *status, cudaStream_t s,
+                                 const float2 *lohi, int n1, int batch, int conj_out, int *status, cudaStream_t s,
                                  int m = 1);  // m > 1: the three-pass form's last pass (no twiddle)
 // middle pass of the three-pass form (m = 2 or 4), in place on the workspace
 cudaError_t launch_fs_mid(float2 *work, const float2 *lohi, int n1, int m, int n3, int batch, cudaStream_t s);

@@ -814,8 +814,8 @@ int run_any(fft_plan_s *p, const float2 *src, float2 *dst, int sign, cudaStream_
 // `in`, out of place into the workspace), pass B (twiddle on load, rows of the
 // workspace, stored transposed into `out`); with m > 1 (2^25, 2^26) an m-point
 // middle pass between them carries the twiddles and pass B's rows are n2 / m
-// long.  The inverse is the forward transform stored at the reflected index
-// (n - k) mod n.
+// long.  The inverse is conj(F(conj x)): pass A conjugates on load, pass B on
+// store.
 int run_fourstep(fft_plan_s *p, const float2 *src, float2 *dst, bool inv, cudaStream_t s) {
     FourStepPlan &fs = p->fs;
     if (fs.map_base != src) {
@@ -824,7 +824,7 @@ int run_fourstep(fft_plan_s *p, const float2 *src, float2 *dst, bool inv, cudaSt
         fs.map_base = src;
     }
     if (p->ev[0] && pass_event(p, 0, s) != cudaSuccess) return FFT_ERR_CUDA;
-    if (launch_cols(*fs.a, fs.map, fs.work, fs.tw_a, fs.n2, p->batch, 1, 0, p->status, fs.grid_a, 0, s) !=
+    if (launch_cols(*fs.a, fs.map, fs.work, fs.tw_a, fs.n2, p->batch, 1, inv ? 2 : 0, p->status, fs.grid_a, 0, s) !=
         cudaSuccess)
         return FFT_ERR_CUDA;
     if (p->ev[1] && pass_event(p, 1, s) != cudaSuccess) return FFT_ERR_CUDA;
