@@ -248,6 +248,137 @@ __global__ void __launch_bounds__(BluShape<N, E>::THREADS, BluShape<N, E>::MINB)
     }
 }
 
+// Bluestein through half-length transforms, one pass.  With M = 2Q and
+// n <= Q only the first half of the padded row is non-zero and only the first
+// half of the inverse is wanted, so the radix-2 level at either end of the
+// length-M convolution needs no partner:
+//     F_M(a)[2k + h] = F_Q(a_j w_M^{h j})[k],                        h = 0, 1
+//     (M F_M^-1 G)[j] = sum_h w_M^{-h j} sum_k G[2k + h] w_Q^{-k j},  j < Q,
+// four length-Q transforms in place of two of length M, in two halves that
+// never meet until their results are added.  Each half of a row's thread
+// group runs one h: chirp in, forward transform, filter product, inverse
+// (as conj(F(conj .))), all on one copy of the engine.  Thread tt holds the
+// elements tt + m*T both as the forward's outputs and as the inverse's
+// inputs, so the two transforms are joined in registers.
+//
+// Tables: c (n chirps); the filter spectrum of half h for k <= Q/2 only,
+// since h[m] = h[M - m] makes H[k] = H[M - k]; and w_M^{tt}, t < T, the rest
+// of w_M^{tt + mT} = w_M^{tt} w_{2E}^m being constants.  Together with the
+// stage twiddles they stay within L1 beside the exchanges.
+//
+// Bound by the shared-memory/L1 pipe (4093 points: 71 % of its wavefronts,
+// half of them the exchanges, half the table reads) and by issue (68 %); DRAM
+// moves one read and one write of the signals.  16384 x 4093: 0.718 ms,
+// against 0.816 for the length-8192 form in two passes over the padded rows;
+// 16627 x 1009: 0.153 / 0.205 (one pass, M = 2048); 4093 x 4099, where M =
+// 16384 took five passes: 0.424 / 1.174.
+struct SyncHalf {  // barrier over the T >= 32 threads of one half (ids from 1)
+    int id, count;
+    __device__ __forceinline__ void operator()() const {
+        asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
+    }
+};
+
+template <int Q, int E>
+struct BluHalfShape {
+    static constexpr int T = Q / E;
+    static constexpr int GROUP = 2 * T;  // threads per row
+    static constexpr int ROWS = GROUP >= 256 ? 1 : 256 / GROUP;
+    static constexpr int THREADS = ROWS * GROUP;
+    static constexpr int MINB = E >= 32 ? 512 / THREADS : T < 32 ? 3 : 1024 / THREADS;
+    using Eng = Engine<Q, E, 1, PadShift<E>::value, RowPadShift1<E>::value>;
+    static constexpr size_t SMEM = sizeof(float2) * 2 * (size_t)ROWS * Eng::SMEM_ELEMS;
+};
+
+template <int Q, int E>
+__global__ void __launch_bounds__(BluHalfShape<Q, E>::THREADS, BluHalfShape<Q, E>::MINB)
+    k_blu_half(const float2 *__restrict__ src, float2 *__restrict__ dst, const float2 *__restrict__ tw,
+               const float2 *__restrict__ chirp, const float2 *__restrict__ Hh, const float2 *__restrict__ wt, int n,
+               long long rows) {
+    using Sh = BluHalfShape<Q, E>;
+    using Eng = typename Sh::Eng;
+    constexpr int T = Sh::T;
+    constexpr int R0 = Eng::R0;
+    constexpr int QS = 32 / E;  // w_{2E} = w_64^QS
+    static_assert(Eng::S > 1 && Eng::SMEM_ELEMS >= Q / 2, "the exchange holds half a row");
+    extern __shared__ __align__(16) float2 smem[];
+    const int grp = threadIdx.x / T;
+    const int h = grp & 1;
+    const int tt = threadIdx.x - grp * T;
+    float2 *sm = smem + grp * Eng::SMEM_ELEMS;
+    const long long row = (long long)blockIdx.x * Sh::ROWS + (grp >> 1);
+    const bool active = row < rows;
+    const float2 w0 = __ldg(wt + (h ? tt : 0));  // w_M^{tt} for the odd half, 1 for the even one
+    auto twist = [&](float2 (&v)[E], auto slot) {  // v[slot(m)] *= w_M^{tt + mT}, the odd half
+#pragma unroll
+        for (int m = 0; m < E; ++m) v[slot(m)] = mul_root64(cmul(v[slot(m)], w0), m * QS);
+    };
+    // register of element tt + m*T in stage-0 order
+    auto in_slot = [](int m) { return (m % (E / R0)) * R0 + m / (E / R0); };
+    auto out_slot = [](int m) { return m; };
+
+    float2 v[E];
+#pragma unroll
+    for (int m = 0; m < E; ++m) {
+        const int i = tt + m * T;
+        v[in_slot(m)] = active && i < n ? __ldg(src + row * n + i) : make_float2(0.f, 0.f);
+    }
+#pragma unroll
+    for (int m = 0; m < E; ++m) {
+        const int i = tt + m * T;
+        v[in_slot(m)] = cmul(v[in_slot(m)], __ldg(chirp + (i < n ? i : n - 1)));
+    }
+    if (h) twist(v, in_slot);
+    auto half_sync = [&] {
+        if constexpr (T >= 32) SyncHalf{1 + grp, T}();
+        else __syncwarp();
+    };
+    // the two transforms as one loop body (two inlined engines are scheduled
+    // into each other and spill)
+#pragma unroll 1
+    for (int ph = 0; ph < 2; ++ph) {
+        float2 u[E];
+        int m_out = 0;
+        Eng::template run<FftPolicy, true>(v, sm, tw, tt, 0, half_sync, [] {},
+                                           [&](int, int, float2 x) { u[m_out++] = x; });
+        if (ph == 0) {
+            const float2 *Hp = Hh + h * (Q / 2 + 1);
+#pragma unroll
+            for (int m = 0; m < E; ++m) {
+                const int k = tt + m * T;
+                const float2 y = cmul(u[m], __ldg(Hp + (m < E / 2 ? k : Q - h - k)));
+                v[in_slot(m)] = make_float2(y.x, -y.y);
+            }
+        } else {
+#pragma unroll
+            for (int m = 0; m < E; ++m) v[m] = u[m];
+        }
+    }
+    if (h) twist(v, out_slot);
+    // the halves add up: each takes half of the elements from the other
+    half_sync();  // the last exchange has been read
+    float2 *mine = sm + tt;
+#pragma unroll
+    for (int m = 0; m < E / 2; ++m) mine[m * T] = h ? v[m] : v[m + E / 2];
+    if constexpr (T >= 32) __syncthreads();
+    else __syncwarp();
+    const float2 *other = smem + (grp ^ 1) * Eng::SMEM_ELEMS + tt;
+#pragma unroll
+    for (int m = 0; m < E / 2; ++m) {
+        const float2 a = h ? v[m + E / 2] : v[m], b = other[m * T];
+        const int i = tt + (m + (h ? E / 2 : 0)) * T;
+        if (active && i < n) dst[row * n + i] = cmul(make_float2(a.x + b.x, -(a.y + b.y)), __ldg(chirp + i));
+    }
+}
+
+// The stored half of both filter spectra: Hh[k] = H[2k], k <= Q/2, then
+// Hh[Q/2 + 1 + k] = H[2k + 1], k < Q/2 (H of length 2Q).
+__global__ void k_blu_half_filter(float2 *Hh, const float2 *__restrict__ H, int Q) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k <= Q / 2) Hh[k] = H[2 * k];
+    if (k < Q / 2) Hh[Q / 2 + 1 + k] = H[2 * k + 1];
+}
+
 namespace {
 BluVariant g_blu[kMaxLog2 + 1];
 std::once_flag g_blu_once;  // registry filled once, safe across host threads
@@ -283,6 +414,36 @@ void init_blu() {
     });
 }
 
+BluHalfVariant g_blu_half[kMaxLog2 + 1];
+std::once_flag g_blu_half_once;
+
+template <int Q>
+void reg_blu_half() {
+    constexpr int E = Q >= 8192 ? 32 : 16;
+    using Sh = BluHalfShape<Q, E>;
+    BluHalfVariant &v = g_blu_half[ilog2(Q)];
+    v.fn = (const void *)k_blu_half<Q, E>;
+    v.q = Q;
+    v.e = E;
+    v.threads = Sh::THREADS;
+    v.rows_per_cta = Sh::ROWS;
+    v.smem = Sh::SMEM;
+}
+// Q = 128 (n = 65 .. 128) is left to the length-M one-pass form: 250406
+// signals of 67 points take 0.256 ms here and 0.236 there (Q = 64, 37 points:
+// 0.207 / 0.261; Q = 256, 251 points: 0.126 / 0.190)
+void init_blu_half() {
+    std::call_once(g_blu_half_once, [] {
+        reg_blu_half<64>();
+        reg_blu_half<256>();
+        reg_blu_half<512>();
+        reg_blu_half<1024>();
+        reg_blu_half<2048>();
+        reg_blu_half<4096>();
+        reg_blu_half<8192>();
+    });
+}
+
 int blocks_for(long long count) {
     long long b = (count + 255) / 256;
     if (b > 152LL * 16) b = 152LL * 16;
@@ -308,6 +469,33 @@ cudaError_t launch_blu(const BluVariant &v, int phase, const float2 *src, float2
     if (grid < 1 || grid > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
     void *args[] = {(void *)&src, (void *)&dst, (void *)&tw, (void *)&chirp, (void *)&H, (void *)&n, (void *)&rows};
     return cudaLaunchKernel(v.fn[phase], dim3((unsigned)grid), dim3(v.threads), args, v.smem, s);
+}
+
+const BluHalfVariant *blu_half_variant(int M) {
+    init_blu_half();
+    if (M < 4 || M > 2 << kMaxLog2 || (M & (M - 1))) return nullptr;
+    const BluHalfVariant *v = &g_blu_half[ilog2(M / 2)];
+    return v->fn ? v : nullptr;
+}
+
+cudaError_t build_blu_half_filter(float2 *Hh, const float2 *H, int q, cudaStream_t s) {
+    k_blu_half_filter<<<(q / 2 + 256) / 256, 256, 0, s>>>(Hh, H, q);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_blu_half(const BluHalfVariant &v, const float2 *src, float2 *dst, const float2 *tw,
+                            const float2 *chirp, const float2 *Hh, const float2 *wt, int n, long long rows,
+                            cudaStream_t s) {
+    if (n < 1 || n > v.q) return cudaErrorInvalidValue;
+    if (v.smem > 48 * 1024) {
+        cudaError_t e = cudaFuncSetAttribute(v.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)v.smem);
+        if (e != cudaSuccess) return e;
+    }
+    const long long grid = (rows + v.rows_per_cta - 1) / v.rows_per_cta;
+    if (grid < 1 || grid > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
+    void *args[] = {(void *)&src, (void *)&dst, (void *)&tw, (void *)&chirp,
+                    (void *)&Hh,  (void *)&wt,  (void *)&n,  (void *)&rows};
+    return cudaLaunchKernel(v.fn, dim3((unsigned)grid), dim3(v.threads), args, v.smem, s);
 }
 
 cudaError_t build_chirp(float2 *c, int n, int sgn, cudaStream_t s) {

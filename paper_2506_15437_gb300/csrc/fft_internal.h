@@ -289,6 +289,20 @@ struct BluVariant {
 const BluVariant *blu_variant(int M);
 cudaError_t launch_blu(const BluVariant &v, int phase, const float2 *src, float2 *dst, const float2 *tw,
                        const float2 *chirp, const float2 *H, int n, long long rows, cudaStream_t s);
+// Bluestein through half-length transforms (fft_bluestein.cu, k_blu_half):
+// padded length M = 2q, signals of n <= q points, one pass.
+struct BluHalfVariant {
+    const void *fn = nullptr;
+    int q = 0, e = 0, threads = 0, rows_per_cta = 0;
+    size_t smem = 0;
+};
+const BluHalfVariant *blu_half_variant(int M);  // nullptr if not compiled
+// Hh: q + 1 entries, the half of both filter spectra that is stored
+cudaError_t build_blu_half_filter(float2 *Hh, const float2 *H, int q, cudaStream_t s);
+// tw: stage twiddles of (q, e); wt: w_M^t, t < q / e
+cudaError_t launch_blu_half(const BluHalfVariant &v, const float2 *src, float2 *dst, const float2 *tw,
+                            const float2 *chirp, const float2 *Hh, const float2 *wt, int n, long long rows,
+                            cudaStream_t s);
 
 // Mixed-radix stages of a 13-smooth length n <= kMixedMaxN (fft_mixed.cu).
 constexpr int kMixedMaxN = 14336;           // two float2 buffers of n in one CTA's shared memory
@@ -350,6 +364,9 @@ struct AnyAxis {
     float2 *mtw = nullptr;              // mixed-radix twiddles (forward)
     const BluVariant *fused = nullptr;  // M <= 8192: fused kernels (same E as the sub-plan's row pass)
     bool fused_one = false;             // the fused transform in one pass (no padded workspace)
+    const BluHalfVariant *half = nullptr;  // the one-pass form over half-length transforms (no sub-plan)
+    float2 *half_tw = nullptr, *half_wt = nullptr;  // its stage twiddles and w_M^t
+    float2 *Hh[2] = {nullptr, nullptr};             // its filter spectra per direction
     int n = 1, M = 0;
     long long rows = 0;
     fft_plan_s *sub = nullptr;           // (n or M, 1, rows), run forward and inverse

@@ -614,8 +614,14 @@ int setup_any_axis(fft_plan_s *p, AnyAxis &ax, int n, long long rows, int cols_n
     }
     ax.M = (int)next_pow2(2LL * n - 1);
     if (rows * ax.M > (1LL << 31)) return FFT_ERR_INVALID_SIZE;
-    ax.sub = create_dense(ax.M, 1, (int)rows, FFT_FORWARD, FFT_PREC_FP32, default_schedule(ax.M, 1), &rc);
-    if (!ax.sub) return rc;
+    const char *ev = getenv("GB300FFT_BLUESTEIN_FUSED");    // 0: the five-pass form (tests, experiments)
+    const char *e1 = getenv("GB300FFT_BLUESTEIN_ONEPASS");  // 0 / 1: the two-pass / one-pass length-M form
+    const bool fused = !(ev && atoi(ev) == 0);
+    if (fused && !e1) ax.half = blu_half_variant(ax.M);
+    if (!ax.half) {
+        ax.sub = create_dense(ax.M, 1, (int)rows, FFT_FORWARD, FFT_PREC_FP32, default_schedule(ax.M, 1), &rc);
+        if (!ax.sub) return rc;
+    }
     for (int d = 0; d < 2; ++d) {
         ax.chirp[d] = dev_alloc<float2>(p, n);
         ax.H[d] = dev_alloc<float2>(p, ax.M);
@@ -633,12 +639,23 @@ int setup_any_axis(fft_plan_s *p, AnyAxis &ax, int n, long long rows, int cols_n
         if (rc == FFT_OK) rc = run_dense(one, filt, ax.H[d], FFT_FORWARD, nullptr, 1.f, 0);
         if (rc == FFT_OK && launch_scale(ax.H[d], ax.M, 1.0f / (float)ax.M, 0) != cudaSuccess) rc = FFT_ERR_CUDA;
     }
+    if (rc == FFT_OK && ax.half) {
+        const int q = ax.half->q, e = ax.half->e;
+        ax.half_tw = dev_alloc<float2>(p, twiddle_table_size(q, e));
+        ax.half_wt = dev_alloc<float2>(p, q / e);
+        for (int d = 0; d < 2; ++d) ax.Hh[d] = dev_alloc<float2>(p, q + 1);
+        if (!ax.half_tw || !ax.half_wt || !ax.Hh[0] || !ax.Hh[1]) rc = FFT_ERR_ALLOC;
+        else if (build_twiddles(ax.half_tw, q, e, 0) != cudaSuccess ||
+                 build_roots_strided(ax.half_wt, q / e, ax.M, 1, 0) != cudaSuccess ||
+                 build_blu_half_filter(ax.Hh[0], ax.H[0], q, 0) != cudaSuccess ||
+                 build_blu_half_filter(ax.Hh[1], ax.H[1], q, 0) != cudaSuccess)
+            rc = FFT_ERR_CUDA;
+    }
     if (rc == FFT_OK && cudaDeviceSynchronize() != cudaSuccess) rc = FFT_ERR_CUDA;
     free_plan(one);
     // fused kernels when the padded length is one row pass with the same E
     // (so they share the sub-plan's twiddle table)
-    const char *ev = getenv("GB300FFT_BLUESTEIN_FUSED");  // 0: the five-pass form (tests, experiments)
-    const BluVariant *fv = (ev && atoi(ev) == 0) ? nullptr : blu_variant(ax.M);
+    const BluVariant *fv = fused && ax.sub ? blu_variant(ax.M) : nullptr;
     if (rc == FFT_OK && fv && ax.sub->rows.row && ax.sub->fs.n1 == 0 && !ax.sub->any &&
         fv->e == ax.sub->rows.row->e && (ax.sub->rows.tw || ax.sub->rows.row->tw_size == 0))
         ax.fused = fv;
@@ -646,9 +663,8 @@ int setup_any_axis(fft_plan_s *p, AnyAxis &ax, int n, long long rows, int cols_n
     // form up to M = 2048 (measured: 0.37 against 0.43 ms for 65536 rows of
     // 500 points, M = 1024), the two-pass one from M = 4096 (0.96 against
     // 0.81 ms for 32768 rows of 2047 points)
-    const char *e1 = getenv("GB300FFT_BLUESTEIN_ONEPASS");  // 0 / 1 forces the form
     ax.fused_one = ax.fused && ax.fused->fn[2] && (e1 ? atoi(e1) != 0 : ax.M <= 2048);
-    if (rc == FFT_OK && !ax.fused_one) {
+    if (rc == FFT_OK && ax.sub && !ax.fused_one) {
         ax.A = dev_alloc<float2>(p, (size_t)rows * ax.M);
         if (!ax.A) return FFT_ERR_ALLOC;
     }
@@ -755,6 +771,11 @@ int run_any_axis(AnyAxis &ax, const float2 *in, float2 *out, int sign, cudaStrea
                                                                                                 : FFT_ERR_CUDA;
     if (!ax.M) return run_dense(ax.sub, in, out, sign, nullptr, 1.f, s);
     const int d = sign > 0 ? 1 : 0;
+    if (ax.half)
+        return launch_blu_half(*ax.half, in, out, ax.half_tw, ax.chirp[d], ax.Hh[d], ax.half_wt, ax.n, ax.rows, s) ==
+                       cudaSuccess
+                   ? FFT_OK
+                   : FFT_ERR_CUDA;
     if (ax.fused) {
         // one pass (each CTA reads its rows before it writes them, so in
         // place is fine), or the two-pass form through the padded rows
@@ -1482,13 +1503,20 @@ int fft_plan_describe(fft_plan_t p, char *buf, int len) {
         k = snprintf(tmp, sizeof tmp, "{\"kind\": \"ragged\", \"kernel\": \"k_ragged\"}");
     } else if (p->any) {
         const gb300fft::AnyPlan &ap = *p->any;
+        // "fused": the length-M Bluestein form of this padded length (0 five
+        // passes, 1 two, 2 one); "half_q" > 0: the one-pass form over
+        // transforms of that length runs in its place
+        auto fused = [](const gb300fft::AnyAxis &ax) {
+            return ax.half ? (ax.M > 8192 ? 0 : ax.M > 2048 ? 1 : 2) : ax.fused ? (ax.fused_one ? 2 : 1) : 0;
+        };
+        auto half = [](const gb300fft::AnyAxis &ax) { return ax.half ? ax.half->q : 0; };
         k = snprintf(tmp, sizeof tmp,
                      "{\"kind\": \"any\", \"precision\": \"fp32\", \"x\": {\"n\": %d, \"bluestein_m\": %d, "
-                     "\"fused\": %d, \"mixed\": %d, \"mixed_fourstep\": [%d, %d]}, \"y\": {\"n\": %d, "
-                     "\"bluestein_m\": %d, \"fused\": %d, \"mixed\": %d, \"mixed_fourstep\": [%d, %d]}, "
+                     "\"fused\": %d, \"half_q\": %d, \"mixed\": %d, \"mixed_fourstep\": [%d, %d]}, \"y\": {\"n\": %d, "
+                     "\"bluestein_m\": %d, \"fused\": %d, \"half_q\": %d, \"mixed\": %d, \"mixed_fourstep\": [%d, %d]}, "
                      "\"transposes\": %d}",
-                     ap.x.n, ap.x.M, ap.x.fused ? (ap.x.fused_one ? 2 : 1) : 0, ap.x.mixed ? 1 : 0, ap.x.n1, ap.x.n2,
-                     ap.y.n, ap.y.M, ap.y.fused ? (ap.y.fused_one ? 2 : 1) : 0, ap.y.mixed ? 1 : 0, ap.y.n1, ap.y.n2,
+                     ap.x.n, ap.x.M, fused(ap.x), half(ap.x), ap.x.mixed ? 1 : 0, ap.x.n1, ap.x.n2,
+                     ap.y.n, ap.y.M, fused(ap.y), half(ap.y), ap.y.mixed ? 1 : 0, ap.y.n1, ap.y.n2,
                      (p->nx > 1 && p->ny > 1 && !ap.y_cols) ? 2 : 0);
     } else if (p->fs.n1 > 0) {
         const gb300fft::FourStepPlan &fs = p->fs;
