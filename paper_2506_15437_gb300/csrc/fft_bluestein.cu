@@ -254,40 +254,54 @@ __global__ void __launch_bounds__(BluShape<N, E>::THREADS, BluShape<N, E>::MINB)
 // length-M convolution needs no partner:
 //     F_M(a)[2k + h] = F_Q(a_j w_M^{h j})[k],                        h = 0, 1
 //     (M F_M^-1 G)[j] = sum_h w_M^{-h j} sum_k G[2k + h] w_Q^{-k j},  j < Q,
-// four length-Q transforms in place of two of length M, in two halves that
-// never meet until their results are added.  Each half of a row's thread
-// group runs one h: chirp in, forward transform, filter product, inverse
-// (as conj(F(conj .))), all on one copy of the engine.  Thread tt holds the
-// elements tt + m*T both as the forward's outputs and as the inverse's
-// inputs, so the two transforms are joined in registers.
+// four length-Q transforms in place of two of length M, in two halves (h)
+// that never meet until their results are added.  A thread carries both
+// halves side by side in the lanes of C2: they share every stage twiddle, so
+// the signal is read once, the butterflies issue as packed instructions and
+// the final sum is within a thread.  Chirp in, forward transform, filter
+// product, inverse (as conj(F(conj .))), chirp out.  Thread tt holds the
+// elements tt + m*T both as the forward's outputs and as the inverse's inputs,
+// so the two transforms are joined in registers.
 //
 // Tables: c (n chirps); the filter spectrum of half h for k <= Q/2 only,
 // since h[m] = h[M - m] makes H[k] = H[M - k]; and w_M^{tt}, t < T, the rest
 // of w_M^{tt + mT} = w_M^{tt} w_{2E}^m being constants.  Together with the
 // stage twiddles they stay within L1 beside the exchanges.
 //
-// Bound by the shared-memory/L1 pipe (4093 points: 71 % of its wavefronts,
-// half of them the exchanges, half the table reads) and by issue (68 %); DRAM
-// moves one read and one write of the signals.  16384 x 4093: 0.718 ms,
-// against 0.816 for the length-8192 form in two passes over the padded rows;
-// 16627 x 1009: 0.153 / 0.205 (one pass, M = 2048); 4093 x 4099, where M =
-// 16384 took five passes: 0.424 / 1.174.
-struct SyncHalf {  // barrier over the T >= 32 threads of one half (ids from 1)
+// The exchange is swizzled, not padded (Engine, kSwizzle): two rows of 4096
+// points are exactly 128 KiB, which leaves an SM enough L1 for all the tables
+// (98 KiB); with padding, or with the signal allocated in L1 as it streams
+// through, two thirds of the table reads went to L2 (hit rate 33 % -> 65 %).
+// Bound by the shared-memory/L1 pipe (65 % of its wavefronts, mostly the
+// exchanges), the FMA pipe (58 %) and, at 16 warps an SM, latency; DRAM moves
+// one read and one write of the signals.  Against the length-M forms this
+// replaces (two passes over padded rows; one pass for M <= 2048; five passes
+// for M = 16384): 16384 x 4093 0.548 / 0.811 ms, 4099 x 4093 0.144 / 0.215, 16627 x 1009
+// 0.130 / 0.205, 32961 x 509 0.121 / 0.192, 4093 x 4099 0.369 / 1.172.  One
+// thread per half instead of one per pair (scalar butterflies, twice the
+// issue slots, halves added through shared memory): 4099 x 4093 0.186.
+struct SyncHalf {  // barrier over the count >= 32 threads of one row (ids from 1)
     int id, count;
     __device__ __forceinline__ void operator()() const {
         asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
     }
 };
 
+// a signal element: read once, so it takes no room in L1 from the tables
+__device__ __forceinline__ float2 ld_stream(const float2 *p) {
+    float2 v;
+    asm("ld.global.nc.L1::no_allocate.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+    return v;
+}
+
 template <int Q, int E>
 struct BluHalfShape {
-    static constexpr int T = Q / E;
-    static constexpr int GROUP = 2 * T;  // threads per row
-    static constexpr int ROWS = GROUP >= 256 ? 1 : 256 / GROUP;
-    static constexpr int THREADS = ROWS * GROUP;
-    static constexpr int MINB = E >= 32 ? 512 / THREADS : T < 32 ? 3 : 1024 / THREADS;
-    using Eng = Engine<Q, E, 1, PadShift<E>::value, RowPadShift1<E>::value>;
-    static constexpr size_t SMEM = sizeof(float2) * 2 * (size_t)ROWS * Eng::SMEM_ELEMS;
+    static constexpr int T = Q / E;  // threads per row
+    static constexpr int ROWS = T >= 256 ? 1 : 256 / T;
+    static constexpr int THREADS = ROWS * T;
+    static constexpr int MINB = (E >= 32 ? 256 : 512) / THREADS;  // 2 E float pairs, and room to work
+    using Eng = Engine<Q, E, 1, kSwizzle>;
+    static constexpr size_t SMEM = sizeof(C2) * (size_t)ROWS * Eng::SMEM_ELEMS;
 };
 
 template <int Q, int E>
@@ -300,74 +314,63 @@ __global__ void __launch_bounds__(BluHalfShape<Q, E>::THREADS, BluHalfShape<Q, E
     constexpr int T = Sh::T;
     constexpr int R0 = Eng::R0;
     constexpr int QS = 32 / E;  // w_{2E} = w_64^QS
-    static_assert(Eng::S > 1 && Eng::SMEM_ELEMS >= Q / 2, "the exchange holds half a row");
-    extern __shared__ __align__(16) float2 smem[];
+    static_assert(Eng::S > 1, "an exchange between the stages");
+    extern __shared__ __align__(16) C2 smem2[];
     const int grp = threadIdx.x / T;
-    const int h = grp & 1;
     const int tt = threadIdx.x - grp * T;
-    float2 *sm = smem + grp * Eng::SMEM_ELEMS;
-    const long long row = (long long)blockIdx.x * Sh::ROWS + (grp >> 1);
+    C2 *sm = smem2 + grp * Eng::SMEM_ELEMS;
+    const long long row = (long long)blockIdx.x * Sh::ROWS + grp;
     const bool active = row < rows;
-    const float2 w0 = __ldg(wt + (h ? tt : 0));  // w_M^{tt} for the odd half, 1 for the even one
-    auto twist = [&](float2 (&v)[E], auto slot) {  // v[slot(m)] *= w_M^{tt + mT}, the odd half
-#pragma unroll
-        for (int m = 0; m < E; ++m) v[slot(m)] = mul_root64(cmul(v[slot(m)], w0), m * QS);
-    };
+    const float2 w0 = __ldg(wt + tt);  // w_M^{tt}
     // register of element tt + m*T in stage-0 order
     auto in_slot = [](int m) { return (m % (E / R0)) * R0 + m / (E / R0); };
-    auto out_slot = [](int m) { return m; };
 
-    float2 v[E];
+    C2 v[E];
+    {
+        float2 x[E];
 #pragma unroll
-    for (int m = 0; m < E; ++m) {
-        const int i = tt + m * T;
-        v[in_slot(m)] = active && i < n ? __ldg(src + row * n + i) : make_float2(0.f, 0.f);
-    }
+        for (int m = 0; m < E; ++m) {
+            const int i = tt + m * T;
+            x[m] = active && i < n ? ld_stream(src + row * n + i) : make_float2(0.f, 0.f);
+        }
 #pragma unroll
-    for (int m = 0; m < E; ++m) {
-        const int i = tt + m * T;
-        v[in_slot(m)] = cmul(v[in_slot(m)], __ldg(chirp + (i < n ? i : n - 1)));
+        for (int m = 0; m < E; ++m) {
+            const int i = tt + m * T;
+            const float2 a = cmul(x[m], __ldg(chirp + (i < n ? i : n - 1)));
+            v[in_slot(m)] = lanes(a, mul_root64(cmul(a, w0), m * QS));
+        }
     }
-    if (h) twist(v, in_slot);
-    auto half_sync = [&] {
-        if constexpr (T >= 32) SyncHalf{1 + grp, T}();
+    auto row_sync = [&] {
+        if constexpr (Sh::ROWS == 1) __syncthreads();
+        else if constexpr (T >= 32) SyncHalf{1 + grp, T}();
         else __syncwarp();
     };
     // the two transforms as one loop body (two inlined engines are scheduled
     // into each other and spill)
 #pragma unroll 1
     for (int ph = 0; ph < 2; ++ph) {
-        float2 u[E];
+        C2 u[E];
         int m_out = 0;
-        Eng::template run<FftPolicy, true>(v, sm, tw, tt, 0, half_sync, [] {},
-                                           [&](int, int, float2 x) { u[m_out++] = x; });
+        Eng::template run<PairPolicy, true>(v, sm, tw, tt, 0, row_sync, [] {},
+                                            [&](int, int, C2 x) { u[m_out++] = x; });
         if (ph == 0) {
-            const float2 *Hp = Hh + h * (Q / 2 + 1);
 #pragma unroll
             for (int m = 0; m < E; ++m) {
                 const int k = tt + m * T;
-                const float2 y = cmul(u[m], __ldg(Hp + (m < E / 2 ? k : Q - h - k)));
-                v[in_slot(m)] = make_float2(y.x, -y.y);
+                const C2 y = cmul(u[m], __ldg(Hh + (m < E / 2 ? k : Q - k)),
+                                  __ldg(Hh + (Q / 2 + 1) + (m < E / 2 ? k : Q - 1 - k)));
+                v[in_slot(m)] = {y.re, make_float2(-y.im.x, -y.im.y)};
             }
         } else {
 #pragma unroll
             for (int m = 0; m < E; ++m) v[m] = u[m];
         }
     }
-    if (h) twist(v, out_slot);
-    // the halves add up: each takes half of the elements from the other
-    half_sync();  // the last exchange has been read
-    float2 *mine = sm + tt;
 #pragma unroll
-    for (int m = 0; m < E / 2; ++m) mine[m * T] = h ? v[m] : v[m + E / 2];
-    if constexpr (T >= 32) __syncthreads();
-    else __syncwarp();
-    const float2 *other = smem + (grp ^ 1) * Eng::SMEM_ELEMS + tt;
-#pragma unroll
-    for (int m = 0; m < E / 2; ++m) {
-        const float2 a = h ? v[m + E / 2] : v[m], b = other[m * T];
-        const int i = tt + (m + (h ? E / 2 : 0)) * T;
-        if (active && i < n) dst[row * n + i] = cmul(make_float2(a.x + b.x, -(a.y + b.y)), __ldg(chirp + i));
+    for (int m = 0; m < E; ++m) {
+        const int i = tt + m * T;
+        const float2 z = cadd(lane_a(v[m]), mul_root64(cmul(lane_b(v[m]), w0), m * QS));
+        if (active && i < n) __stcs(dst + row * n + i, cmul(make_float2(z.x, -z.y), __ldg(chirp + i)));
     }
 }
 
@@ -419,6 +422,8 @@ std::once_flag g_blu_half_once;
 
 template <int Q>
 void reg_blu_half() {
+    // 8192 points with E = 16 would take a third exchange (0.498 against 0.402
+    // ms for 4093 x 4099, before the swizzle)
     constexpr int E = Q >= 8192 ? 32 : 16;
     using Sh = BluHalfShape<Q, E>;
     BluHalfVariant &v = g_blu_half[ilog2(Q)];
@@ -429,12 +434,12 @@ void reg_blu_half() {
     v.rows_per_cta = Sh::ROWS;
     v.smem = Sh::SMEM;
 }
-// Q = 128 (n = 65 .. 128) is left to the length-M one-pass form: 250406
-// signals of 67 points take 0.256 ms here and 0.236 there (Q = 64, 37 points:
-// 0.207 / 0.261; Q = 256, 251 points: 0.126 / 0.190)
+// from Q = 64: 541200 signals of 31 points (Q = 32) take 0.194 ms here and
+// 0.162 in the length-M one-pass form; 275036 of 61 points 0.132 and 0.174
 void init_blu_half() {
     std::call_once(g_blu_half_once, [] {
         reg_blu_half<64>();
+        reg_blu_half<128>();
         reg_blu_half<256>();
         reg_blu_half<512>();
         reg_blu_half<1024>();

@@ -99,19 +99,97 @@ __host__ __device__ constexpr int bitrev(int k, int bits) {
     return bits == 0 ? 0 : ((k & 1) << (bits - 1)) | bitrev(k >> 1, bits - 1);
 }
 
+// ---------------------------------------------------------------------------
+// Two independent complex values side by side, one per lane of the packed
+// float32 instructions (fma/add/mul .f32x2): re = (re_a, re_b), im = (im_a,
+// im_b).  A packed instruction does two lanes in one issue slot at the same
+// lane rate, so kernels bound by issue run the same butterflies over C2 --
+// two transforms that share every twiddle -- in half the slots.  Keeping real
+// and imaginary parts in separate registers (not (re, im) packed) leaves every
+// complex operation lane-wise: no swaps, and each product is the same
+// multiply-add as the scalar form's.
+// ---------------------------------------------------------------------------
+struct __align__(16) C2 {
+    float2 re, im;
+};
+
+__device__ __forceinline__ unsigned long long f2_bits(float2 a) {
+    unsigned long long u;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(u) : "f"(a.x), "f"(a.y));
+    return u;
+}
+__device__ __forceinline__ float2 f2_from(unsigned long long u) {
+    float2 a;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a.x), "=f"(a.y) : "l"(u));
+    return a;
+}
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+    unsigned long long d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(f2_bits(a)), "l"(f2_bits(b)), "l"(f2_bits(c)));
+    return f2_from(d);
+}
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
+    unsigned long long d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(f2_bits(a)), "l"(f2_bits(b)));
+    return f2_from(d);
+}
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+    unsigned long long d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(f2_bits(a)), "l"(f2_bits(b)));
+    return f2_from(d);
+}
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) {
+    unsigned long long d;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(f2_bits(a)), "l"(f2_bits(b)));
+    return f2_from(d);
+}
+__device__ __forceinline__ float2 both(float a) { return make_float2(a, a); }
+
+__device__ __forceinline__ C2 cadd(C2 a, C2 b) { return {add2(a.re, b.re), add2(a.im, b.im)}; }
+__device__ __forceinline__ C2 csub(C2 a, C2 b) { return {sub2(a.re, b.re), sub2(a.im, b.im)}; }
+// both lanes times one complex value
+__device__ __forceinline__ C2 cmul(C2 a, float2 w) {
+    const float2 wr = both(w.x);
+    return {fma2(a.im, both(-w.y), mul2(a.re, wr)), fma2(a.im, wr, mul2(a.re, both(w.y)))};
+}
+// lane a times wa, lane b times wb
+__device__ __forceinline__ C2 cmul(C2 a, float2 wa, float2 wb) {
+    const float2 wr = make_float2(wa.x, wb.x);
+    return {fma2(a.im, make_float2(-wa.y, -wb.y), mul2(a.re, wr)),
+            fma2(a.im, wr, mul2(a.re, make_float2(wa.y, wb.y)))};
+}
+__device__ __forceinline__ float2 lane_a(C2 v) { return make_float2(v.re.x, v.im.x); }
+__device__ __forceinline__ float2 lane_b(C2 v) { return make_float2(v.re.y, v.im.y); }
+__device__ __forceinline__ C2 lanes(float2 a, float2 b) { return {make_float2(a.x, b.x), make_float2(a.y, b.y)}; }
+
+// (u - v) * exp(-2*pi*i*q/64), 0 <= q < 32 a constant after unrolling
+__device__ __forceinline__ float2 sub_root64(float2 u, float2 v, int q) { return mul_root64(csub(u, v), q); }
+__device__ __forceinline__ C2 sub_root64(C2 u, C2 v, int q) {
+    if (q == 16) return {sub2(u.im, v.im), sub2(v.re, u.re)};  // times -i: no negation left over
+    const C2 d = csub(u, v);
+    if (q == 0) return d;
+    if (q == 8 || q == 24) {
+        const float h = 0.7071067811865475f;
+        const float2 sum = add2(d.re, d.im), dif = sub2(d.im, d.re);
+        return q == 8 ? C2{mul2(sum, both(h)), mul2(dif, both(h))} : C2{mul2(dif, both(h)), mul2(sum, both(-h))};
+    }
+    const float c = cos64(q), s = sin64(q);
+    return {fma2(d.im, both(s), mul2(d.re, both(c))), fma2(d.re, both(-s), mul2(d.im, both(c)))};
+}
+
 // One radix-2 decimation-in-frequency level of span H over R registers:
 // (u, v) -> (u + v, (u - v) * w_{2H}^k).  Levels recurse at compile time so
 // every register index and twiddle is a constant.
-template <int R, int H>
-__device__ __forceinline__ void dif_level(float2 *a) {
+template <int R, int H, class V>
+__device__ __forceinline__ void dif_level(V *a) {
     if constexpr (H >= 1) {
 #pragma unroll
         for (int blk = 0; blk < R; blk += 2 * H) {
 #pragma unroll
             for (int k = 0; k < H; ++k) {
-                const float2 u = a[blk + k], v = a[blk + k + H];
+                const V u = a[blk + k], v = a[blk + k + H];
                 a[blk + k] = cadd(u, v);
-                a[blk + k + H] = mul_root64(csub(u, v), k * (64 / (2 * H)));
+                a[blk + k + H] = sub_root64(u, v, k * (64 / (2 * H)));
             }
         }
         dif_level<R, H / 2>(a);
@@ -119,8 +197,8 @@ __device__ __forceinline__ void dif_level(float2 *a) {
 }
 
 // a[K] = t[bitrev(K)] for K = 0..R-1, every index a constant expression.
-template <int R, int K>
-__device__ __forceinline__ void bitrev_gather(float2 *a, const float2 *t) {
+template <int R, int K, class V>
+__device__ __forceinline__ void bitrev_gather(V *a, const V *t) {
     if constexpr (K < R) {
         constexpr int src = bitrev(K, ilog2(R));
         a[K] = t[src];
@@ -131,11 +209,11 @@ __device__ __forceinline__ void bitrev_gather(float2 *a, const float2 *t) {
 // In-register length-R DFT (forward sign), natural order in and out,
 // R a power of two <= 64: radix-2 DIF levels, then a compile-time
 // bit-reversal of register names.
-template <int R>
-__device__ __forceinline__ void dft(float2 *a) {
+template <int R, class V>
+__device__ __forceinline__ void dft(V *a) {
     if constexpr (R > 1) {
         dif_level<R, R / 2>(a);
-        float2 t[R];
+        V t[R];
 #pragma unroll
         for (int k = 0; k < R; ++k) t[k] = a[k];
         bitrev_gather<R, 0>(a, t);
@@ -174,6 +252,14 @@ struct FftPolicy {
     __device__ __forceinline__ void butterfly(T *a) const { dft<R>(a); }
     __device__ __forceinline__ T twiddle(T a, float2 w) const { return cmul(a, w); }
 };
+// two transforms per thread, one per lane of C2
+struct PairPolicy {
+    using T = C2;
+    static constexpr bool kUsesTwiddles = true;
+    template <int R>
+    __device__ __forceinline__ void butterfly(T *a) const { dft<R>(a); }
+    __device__ __forceinline__ T twiddle(T a, float2 w) const { return cmul(a, w); }
+};
 struct MovePolicy {
     using T = float2;  // integer tags carried bit-for-bit in the .x lane
     static constexpr bool kUsesTwiddles = false;
@@ -202,6 +288,8 @@ struct SyncWarp {
 // SRC_IN_SMEM: stage-0 inputs were read from `sm` itself, so the first
 // shared-memory write must wait for every thread's reads.
 // ---------------------------------------------------------------------------
+constexpr int kSwizzle = 31;  // Engine's PADSH: xor swizzle in place of padding
+
 template <int N, int E, int W, int PADSH, int PADSH1 = PADSH>
 struct Engine {
     using Sc = Sched<N, E>;
@@ -214,8 +302,18 @@ struct Engine {
     // use its own shift (PADSH1), since its write pattern follows radix R0
     __host__ __device__ static constexpr int pad(int f) { return f + (f >> PADSH); }
     __host__ __device__ static constexpr int pad_s(int f, int s) { return f + (f >> (s == 1 ? PADSH1 : PADSH)); }
+    // PADSH = kSwizzle: no padding; the low three bits of the index are
+    // xored with higher ones instead (16-byte elements, eight to a row of
+    // banks): every write and read below is then conflict-free over the eight
+    // lanes of a quarter-warp, and the buffer is exactly N*W elements
+    static constexpr bool SWZ = PADSH == kSwizzle;
+    __host__ __device__ static constexpr int swz(int f, int s) {
+        return f ^ ((f >> (s == 1 && R0 < 16 ? 3 : 4)) & 7);
+    }
     static constexpr int SMEM_ELEMS =
-        (S > 1) ? (pad_s(N * W - 1, 1) > pad(N * W - 1) ? pad_s(N * W - 1, 1) : pad(N * W - 1)) + 1 : 0;
+        (S == 1) ? 0
+        : SWZ    ? N * W
+                 : (pad_s(N * W - 1, 1) > pad(N * W - 1) ? pad_s(N * W - 1, 1) : pad(N * W - 1)) + 1;
 
     template <class Pol, bool SRC_IN_SMEM, class Sync, class AfterReads, class Store>
     __device__ static __forceinline__ void run(typename Pol::T (&v)[E], typename Pol::T *sm,
@@ -246,13 +344,24 @@ struct Engine {
                     const int j = tt + b * T;
                     const int m = j & (Nsp - 1);
 #pragma unroll
-                    for (int k = 0; k < Rp; ++k) sm[pad_s(((j - m) * Rp + m + k * Nsp) * W + c, s)] = v[b * Rp + k];
+                    for (int k = 0; k < Rp; ++k) {
+                        // the swizzle is linear over xor, and k*Nsp (below:
+                        // r*T) has no bit in common with the rest: its part
+                        // of the index is a constant
+                        if constexpr (SWZ)
+                            sm[swz(((j - m) * Rp + m) * W + c, s) ^ swz(k * Nsp * W, s)] = v[b * Rp + k];
+                        else
+                            sm[pad_s(((j - m) * Rp + m + k * Nsp) * W + c, s)] = v[b * Rp + k];
+                    }
                 }
                 sync();
                 const int Ns = Sc::ns(s);
                 const int m = tt & (Ns - 1);
 #pragma unroll
-                for (int r = 0; r < E; ++r) v[r] = sm[pad_s((tt + r * T) * W + c, s)];
+                for (int r = 0; r < E; ++r) {
+                    if constexpr (SWZ) v[r] = sm[swz(tt * W + c, s) ^ swz(r * T * W, s)];
+                    else v[r] = sm[pad_s((tt + r * T) * W + c, s)];
+                }
                 if (s == S - 1) after_reads();
                 if constexpr (Pol::kUsesTwiddles) {
                     // twiddles r = 2k+1, 2k+2 of this butterfly in one 16-byte load

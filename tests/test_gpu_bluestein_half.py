@@ -1,5 +1,5 @@
 """The one-pass Bluestein kernel over half-length transforms (padded length
-M = 2Q, Q = 64, 256 ... 8192) against the FP64 oracle, at the shortest and longest
+M = 2Q, Q = 64 ... 8192) against the FP64 oracle, at the shortest and longest
 lengths each Q takes, with a last CTA that is partly filled, both directions
 and in place.
 
@@ -28,7 +28,7 @@ def g():
     return g
 
 
-LENGTHS = [n for q in (64, 256, 512, 1024, 2048, 4096, 8192) for n in (q // 2 + 1, q - 1)]
+LENGTHS = [n for q in (64, 128, 256, 512, 1024, 2048, 4096, 8192) for n in (q // 2 + 1, q - 1)]
 
 
 @pytest.mark.parametrize("n", LENGTHS)
