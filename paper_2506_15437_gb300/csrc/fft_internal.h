@@ -304,20 +304,24 @@ cudaError_t launch_blu_half(const BluHalfVariant &v, const float2 *src, float2 *
                             const float2 *chirp, const float2 *Hh, const float2 *wt, int n, long long rows,
                             cudaStream_t s);
 
-// Mixed-radix stages of a 13-smooth length n <= kMixedMaxN (fft_mixed.cu).
-constexpr int kMixedMaxN = 14336;           // two float2 buffers of n in one CTA's shared memory
+// Mixed-radix stages of a 13-smooth length n <= kMixedMaxN (fft_mixed.cu,
+// fft_mixed_pair.cuh); mixed_factor fills n, S and radix only.
+constexpr int kMixedMaxN = 14336;           // one buffer of pairs in one CTA's shared memory
 constexpr size_t kMixedMaxSmem = 227 * 1024;
 constexpr int kMixedMaxStages = 16;
 struct MixedStages {
     int n = 0, S = 0, tw_size = 0;
-    int wlog = 0;                      // log2 of the columns per CTA (column kernel)
-    int buf_elems = 0;                 // elements of one padded shared-memory buffer
-    int pad[kMixedMaxStages] = {};     // padding shift of the buffer stage s writes (0: none)
+    int wlog = 0;                      // log2 of the elements (transforms, or pairs) per position
+    int buf_elems = 0;                 // buffer elements per transform (pair)
+    int skew = 0;                      // elements left out after each block of one k_0
     int radix[kMixedMaxStages] = {};
-    int ns[kMixedMaxStages] = {};      // product of the radices before stage s
+    int ns[kMixedMaxStages] = {};      // product of the radices after stage s
     int nb[kMixedMaxStages] = {};      // butterflies per transform, n / radix
-    uint32_t mag_nb[kMixedMaxStages] = {}, mag_ns[kMixedMaxStages] = {};  // ceil(2^32 / d) divisors
-    int tw_off[kMixedMaxStages] = {};  // stage s's twiddles w_{Ns R}^{k r}, 16-byte pairs (r odd, r + 1) at pair (r - 1) / 2 * Ns + k
+    int kdiv[kMixedMaxStages] = {};    // radix[1] ... radix[s - 1]
+    // ceil(2^32 / d) divisors by nb, ns, radix and kdiv
+    uint32_t mag_nb[kMixedMaxStages] = {}, mag_ns[kMixedMaxStages] = {}, mag_r[kMixedMaxStages] = {},
+             mag_k[kMixedMaxStages] = {};
+    int tw_off[kMixedMaxStages] = {};  // stage s's twiddles w_{ns R}^{q r}, 16-byte pairs (r odd, r + 1) at pair (r - 1) / 2 * ns + q
 };
 // Second pass of a mixed-radix four-step transform (n = n1 n2): row k1 of
 // the first pass's output is multiplied by w_n^{i2 k1} as it is loaded and
@@ -329,23 +333,31 @@ struct FourStepB {
     int lshift = 0, lmask = 0;
 };
 
-// Launch configuration of the mixed-radix kernel for one axis, fixed at
-// plan creation: transforms per CTA, threads, padded buffers.
+// Launch configuration of the mixed-radix kernels for one axis, fixed at
+// plan creation: kernel, transforms per CTA, threads, schedule.
 struct MixedLaunch {
     MixedStages m;
+    int rmax = 0;  // largest radix compiled into the kernel over pairs; 0: the one-transform kernel
     bool cols = false;
     int nx = 0;  // columns: row length of the [ny][nx] slices
-    int W = 1, T = 0;
+    int W = 2, T = 0;
+    int T_most = 0;  // threads that run every stage in one round
     size_t smem = 0;
     FourStepB fs;
 };
+// The kernels (fft_mixed_pair.cuh), compiled per largest radix: threads whose
+// registers fill an SM (96 and 128 each).
+constexpr int mixed_pair_threads(int rmax) { return rmax <= 13 ? 640 : 512; }
+const void *mixed_pair13_fn(bool cols, bool fs);
+const void *mixed_pair16_fn(bool cols, bool fs);
+constexpr int kMixedOneThreads = 1024;  // of 64 registers
+const void *mixed_one_fn(bool cols, bool fs);
 bool mixed_factor(int n, MixedStages *st);  // false unless n = 2^a 3^b 5^c 7^d 11^e 13^f <= kMixedMaxN
 cudaError_t build_mixed_twiddles(float2 *tw, const MixedStages &st, cudaStream_t s);
-int mixed_rows_per_cta(int n);
-int mixed_cols_width(int n, int nx);
-// 0 on success; fs_n1 > 0: the second pass of a four-step transform with
-// n1 rows per transform (rows layout)
-int mixed_prepare(const MixedStages &st, bool cols, int nx, MixedLaunch *out, int fs_n1 = 0);
+// 0 on success; `count` transforms in all; fourstep: a pass of a four-step
+// transform, the second one (rows layout) with fs_n1 > 0 rows per transform
+int mixed_prepare(const MixedStages &st, bool cols, int nx, long long count, MixedLaunch *out, bool fourstep = false,
+                  int fs_n1 = 0);
 // n = n1 n2 with both factors mixed-radix lengths (<= kMixedMaxN), n1 and
 // n2 as close as possible; false if none
 bool mixed_split(int n, int *n1, int *n2);

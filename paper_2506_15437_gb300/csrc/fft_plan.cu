@@ -579,10 +579,11 @@ int setup_any_axis(fft_plan_s *p, AnyAxis &ax, int n, long long rows, int cols_n
     }
     if (use_mixed(n, &ax.mst)) {
         ax.mixed = true;
-        ax.mtw = dev_alloc<float2>(p, ax.mst.tw_size > 0 ? ax.mst.tw_size : 1);
+        if (mixed_prepare(ax.mst, cols_nx > 0, cols_nx, rows, &ax.ml) != 0) return FFT_ERR_UNSUPPORTED;
+        const MixedStages &m = ax.ml.m;  // the stages of the kernel chosen
+        ax.mtw = dev_alloc<float2>(p, m.tw_size > 0 ? m.tw_size : 1);
         if (!ax.mtw) return FFT_ERR_ALLOC;
-        if (mixed_prepare(ax.mst, cols_nx > 0, cols_nx, &ax.ml) != 0) return FFT_ERR_UNSUPPORTED;
-        return build_mixed_twiddles(ax.mtw, ax.mst, 0) == cudaSuccess ? FFT_OK : FFT_ERR_CUDA;
+        return build_mixed_twiddles(ax.mtw, m, 0) == cudaSuccess ? FFT_OK : FFT_ERR_CUDA;
     }
     // a longer smooth length: four-step over two mixed-radix passes (columns
     // of length n1 into a workspace, then rows of length n2 with the
@@ -590,18 +591,20 @@ int setup_any_axis(fft_plan_s *p, AnyAxis &ax, int n, long long rows, int cols_n
     if (use_mixed_fourstep(n, &ax.n1, &ax.n2)) {
         MixedStages sa, sb;
         if (!mixed_factor(ax.n1, &sa) || !mixed_factor(ax.n2, &sb)) return FFT_ERR_UNSUPPORTED;
-        if (mixed_prepare(sa, true, ax.n2, &ax.mla) != 0 || mixed_prepare(sb, false, 0, &ax.mlb, ax.n1) != 0)
+        if (mixed_prepare(sa, true, ax.n2, rows * ax.n2, &ax.mla, true) != 0 ||
+            mixed_prepare(sb, false, 0, rows * ax.n1, &ax.mlb, true, ax.n1) != 0)
             return FFT_ERR_UNSUPPORTED;
         int lshift = 0;
         while ((1LL << (2 * lshift)) < n) ++lshift;  // 2^lshift >= sqrt(n)
         const int nlo = 1 << lshift, nhi = (int)((n + nlo - 1) / nlo);
-        ax.mtwa = dev_alloc<float2>(p, sa.tw_size > 0 ? sa.tw_size : 1);
-        ax.mtwb = dev_alloc<float2>(p, sb.tw_size > 0 ? sb.tw_size : 1);
+        const MixedStages &ma = ax.mla.m, &mb = ax.mlb.m;  // the stages of the kernels chosen
+        ax.mtwa = dev_alloc<float2>(p, ma.tw_size > 0 ? ma.tw_size : 1);
+        ax.mtwb = dev_alloc<float2>(p, mb.tw_size > 0 ? mb.tw_size : 1);
         ax.fs_lo = dev_alloc<float2>(p, nlo);
         ax.fs_hi = dev_alloc<float2>(p, nhi);
         ax.fs_work = dev_alloc<float2>(p, (size_t)rows * n);
         if (!ax.mtwa || !ax.mtwb || !ax.fs_lo || !ax.fs_hi || !ax.fs_work) return FFT_ERR_ALLOC;
-        if (build_mixed_twiddles(ax.mtwa, sa, 0) != cudaSuccess || build_mixed_twiddles(ax.mtwb, sb, 0) != cudaSuccess ||
+        if (build_mixed_twiddles(ax.mtwa, ma, 0) != cudaSuccess || build_mixed_twiddles(ax.mtwb, mb, 0) != cudaSuccess ||
             build_roots_strided(ax.fs_lo, nlo, n, 1, 0) != cudaSuccess ||
             build_roots_strided(ax.fs_hi, nhi, n, nlo, 0) != cudaSuccess)
             return FFT_ERR_CUDA;
