@@ -22,7 +22,10 @@ template <int N, int E, int W>
 struct ColShape {
     static constexpr int T = N / E;
     static constexpr int THREADS = T * W;
-    static constexpr int MINB = THREADS >= 512 ? (E >= 32 ? 512 : 1024) / THREADS : (THREADS >= 256 && E < 32 ? 3 : 1);
+    // E = 32 below 4096 points, E = 64 at 2048: the registers of 512 and 256 threads an SM
+    static constexpr int FIT = (E >= 64 ? 256 : 512) / THREADS;
+    static constexpr int MINB = (N < 4096 && E >= 32) ? (FIT > 0 ? FIT : 1)
+                                : THREADS >= 512 ? (E >= 32 ? 512 : 1024) / THREADS : (THREADS >= 256 && E < 32 ? 3 : 1);
     using Eng = Engine<N, E, W, PadShift<E>::value>;
     static constexpr int ELEMS = Eng::SMEM_ELEMS > N * W ? Eng::SMEM_ELEMS : N * W;
     static constexpr int BOXR = N < 256 ? N : 256;
@@ -330,7 +333,7 @@ void reg_col(int eslot) {
     en.v.box_rows = Sh::BOXR;
     en.v.tw_size = Sched<N, E>::tw_size;
     en.movemap = (const void *)k_cols_movemap<N, E, W>;
-    if constexpr (N >= 32 && N <= 2048 && THREADS_OK<N, E, W>::value) en.wadj = (const void *)k_cols_wadj<N, E, W>;
+    if constexpr (N >= 32 && N <= 2048 && E <= 16 && THREADS_OK<N, E, W>::value) en.wadj = (const void *)k_cols_wadj<N, E, W>;
 }
 
 template <int N, int E>
@@ -345,8 +348,8 @@ template <int N>
 void reg_cols_n() {
     constexpr int E = N >= 16 ? 16 : N;
     reg_col_ws<N, E>(0);
-    if constexpr (N >= 4096) reg_col_ws<N, 32>(1);
-    if constexpr (N >= 4096) reg_col_ws<N, 64>(2);
+    if constexpr (N >= 4096 || N == 512 || N == 1024) reg_col_ws<N, 32>(1);
+    if constexpr (N >= 2048) reg_col_ws<N, 64>(2);
 }
 
 void init_cols() {
@@ -383,27 +386,39 @@ const ColEntry *col_entry(int log2n, int e, int w) {
 int default_col_e(int n) { return n >= 16 ? 16 : n; }
 
 // Elements per thread the column pass prefers for length n and tile width w:
-// E = 64 makes a 4096-point column two stages with one shared-memory
-// exchange, so the tile is free for the next TMA copy after half the work
-// (measured 0.35 -> 0.26 ms for the 8192^2 column pass).
+// the fewest that make the transform two stages with one shared-memory
+// exchange (512 = 16 32, 1024 = 32 32, 2048 = 32 64, 4096 = 64 64).  Half the
+// exchanges and barriers, and the tile is free for the next TMA copy after half
+// the work, outweigh the fewer warps: 2^24 points, E = 16 against these: 64 x
+// 512^2 0.061 -> 0.049 ms, 16 x 1024^2 0.068 -> 0.053, 4 x 2048^2 0.069 ->
+// 0.059 (8192^2 in 4096-point blocks 0.35 -> 0.26).
 int preferred_col_e(int n, int w) {
-    if (n == 4096 && col_variant(ilog2(n), 64, w)) return 64;
-    return default_col_e(n);
+    const int e = n == 512 || n == 1024 ? 32 : n == 2048 || n == 4096 ? 64 : default_col_e(n);
+    return col_variant(ilog2(n), e, w) ? e : default_col_e(n);
 }
 
-// Widest tile that keeps the staged tile within 128 KiB (columns of 4096
+// Widest tile that keeps the staged tile within 128 KiB (columns of 2048
 // points and more) or 64 KiB (shorter columns: two CTAs per SM, one
 // transforming while the other loads; measured against 128 KiB tiles,
-// 4 x 2048^2 0.136 -> 0.127 ms, 16 x 1024^2 0.124 -> 0.119) and the row
-// length: rows of at least 32 bytes (W >= 4) make whole DRAM sectors, which
-// the TMA moves far faster than 16-byte rows.
+// 16 x 1024^2 0.059 -> 0.053 ms) and the row length: rows of at least 32 bytes
+// (W >= 4) make whole DRAM sectors, which the TMA moves far faster than
+// 16-byte rows.  (2048 points with E = 64: 8 columns 0.119 ms for 8 x 2048^2, 4
+// columns 0.123.)
 int default_col_w(int n, int nx) {
-    int w = (n >= 4096 ? 16384 : 8192) / n;
+    int w = (n >= 2048 ? 16384 : 8192) / n;
     if (w > 16) w = 16;
     if (w < 2) w = 2;
     while (w > nx) w >>= 1;
     return w;
 }
+
+// Tiles ahead that the column pass asks L2 for, `per_cta` tiles to a CTA:
+// 128-point columns finish a tile sooner than the next one lands (1024 x 128^2,
+// 18 tiles to a CTA: 0.055 -> 0.045 ms); with few tiles to a CTA the first
+// requests only delay the first tiles (8 x 128 x 4096, 4 tiles: 0.0142 ->
+// 0.0159), and longer columns lose by it (1024 points 0.053 -> 0.055, 4096
+// 0.246 -> 0.294).
+int default_col_pf(int n, long long per_cta) { return n == 128 && per_cta >= 8 ? 1 : 0; }
 
 const ColVariant *col_variant(int log2n, int e, int w) {
     const ColEntry *en = col_entry(log2n, e, w);

@@ -62,8 +62,9 @@ struct FsRowShape {
     static constexpr size_t BAR_OFF = (G_OFF + (size_t)W * GROW * sizeof(float2) + 15) / 16 * 16;
     static constexpr size_t SMEM = BAR_OFF + 16;
     static constexpr uint32_t TILE_BYTES = (uint32_t)W * N * sizeof(float2);
-    // E = 16: cap at 64 registers (several CTAs per SM); larger E: one CTA
-    static constexpr int MINB_RAW = E <= 16 ? 1024 / THREADS : 1;
+    // E = 16: cap at 64 registers (several CTAs per SM); E = 32 and 64 below
+    // 4096 points: the registers of 512 and 256 threads an SM; else one CTA
+    static constexpr int MINB_RAW = E <= 16 ? 1024 / THREADS : N >= 4096 ? 1 : (E >= 64 ? 256 : 512) / THREADS;
     static constexpr int MINB = MINB_RAW < 1 ? 1 : (MINB_RAW > 32 ? 32 : MINB_RAW);
 };
 
@@ -203,6 +204,15 @@ void reg_fs_row_ws() {
     reg_fs_row<N, 16, 4>();
     reg_fs_row<N, 16, 8>();
     if constexpr (N <= 1024) reg_fs_row<N, 16, 16>();
+    if constexpr (N == 512 || N == 1024) {
+        reg_fs_row<N, 32, 4>();
+        reg_fs_row<N, 32, 8>();
+        reg_fs_row<N, 32, 16>();
+    }
+    if constexpr (N == 2048) {
+        reg_fs_row<N, 64, 4>();
+        reg_fs_row<N, 64, 8>();
+    }
 }
 void init_fs_rows() {
     std::call_once(g_fs_rows_once, [] {
@@ -220,14 +230,17 @@ void init_fs_rows() {
 }
 }  // namespace
 
-// Elements per thread pass B prefers for row length n: 64 at 4096 (one
-// shared-memory exchange), 32 at 8192 (two), otherwise 16.
-int fourstep_row_e(int n) { return n == 4096 ? 64 : n == 8192 ? 32 : 16; }
+// Elements per thread pass B prefers for row length n: as in the column pass,
+// the fewest that leave one shared-memory exchange (2^24 points, E = 16 against
+// these: 512-point rows 0.068 -> 0.059 ms, 1024 0.080 -> 0.056, 2048 0.080 ->
+// 0.074); 32 at 8192 (two exchanges), 16 otherwise.
+int fourstep_row_e(int n) { return n == 4096 || n == 2048 ? 64 : n == 8192 || n == 1024 || n == 512 ? 32 : 16; }
 
-// Rows per CTA pass B prefers for row length n: 4 (32-byte store chunks;
-// measured fastest from 256 to 4096), 8 at 128, 2 at 8192 (the exchange
-// buffer's limit).
-int fourstep_row_w(int n) { return n >= 8192 ? 2 : n <= 128 ? 8 : 4; }
+// Rows per CTA pass B prefers for row length n: 8 (64-byte store chunks; 256
+// points 0.053 -> 0.049 ms against 4), 4 where 8 rows fill too much of an SM
+// (4096) or measured slower (1024: 0.058 against 0.056), 2 at 8192 (the
+// exchange buffer's limit).
+int fourstep_row_w(int n) { return n >= 8192 ? 2 : n == 4096 || n == 1024 ? 4 : 8; }
 
 const ColVariant *fourstep_row_variant(int log2n, int e, int w) {
     init_fs_rows();

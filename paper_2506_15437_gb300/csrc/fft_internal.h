@@ -45,6 +45,7 @@ bool row_variant_info(int n, int e, int split, int *threads, int *rows_per_cta, 
 int default_col_e(int n);
 int preferred_col_e(int n, int w);
 int default_col_w(int n, int nx);
+int default_col_pf(int n, long long per_cta);
 
 // Stage radices of the (n, e) schedule, first stage first; returns count.
 int schedule_radices(int n, int e, int *radices);
@@ -223,7 +224,7 @@ struct Schedule {
     int col_e = 0;         // elements per thread of the column pass (0: default)
     int col_w = 0;         // TMA tile width (0: default)
     int col_c = 2;         // cluster size of the DSMEM column kernel
-    int col_pf = 0;        // TMA column pass: L2 prefetch distance (tiles)
+    int col_pf = -1;       // TMA column pass: L2 prefetch distance (tiles; -1: by length)
     int col_stream = 1;    // out-of-place calls: streaming column pass over row-permuted rows, where compiled
     int col_tstore = 1;    // streaming column pass through TMA stores: 1 unsplit blocks, 2 always, 0 never
     int planar = 1;        // pre-split plans with the streaming pass: blocks as planes of a workspace
@@ -239,6 +240,7 @@ struct AxisPlan {
     float2 *tw = nullptr;
     int n = 1;
     int grid = 0;  // column pass: persistent grid size
+    int pf = 0;    // column pass: L2 prefetch distance in tiles
     int tc_w = 0;  // tensor-core column pass: tile width
     int tcg = 0;   // tensor-core column pass: 1 tcgen05 butterflies, 0 mma.sync
     int tc32 = 0;  // tensor-core pass with radix-32 tcgen05 stages (rows: the plan's rows axis)
@@ -444,7 +446,6 @@ struct fft_plan_s {
     bool ring = false;    // long rows: TMA landing-ring row kernel
     int row_persist = -1;  // row pass grid: 1 persistent, 0 one CTA per group, -1 persistent iff split
     int row_pf = 1;        // persistent row pass: L2 prefetch distance in groups
-    int col_pf = 0;        // column pass: L2 prefetch distance in tiles (0: measured best)
     int *status = nullptr;  // device status word
     void *w16 = nullptr;    // split-FP16 plans: hi/lo W16 table (FP64-built)
     void *w32 = nullptr;    // split-FP16 plans with radix-32 stages: hi/lo B table (FP64-built)

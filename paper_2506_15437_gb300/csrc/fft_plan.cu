@@ -72,7 +72,7 @@ const ColVariant *wadj_variant(fft_plan_s *p) {
     if (n > 2048 || !is_pow2(n)) return nullptr;
     int w = default_col_w(n, p->nx);
     while (w > 2 && (long long)n * w * sizeof(float2) > 65536) w >>= 1;
-    const ColVariant *v = col_variant(ilog2(n), preferred_col_e(n, w), w);
+    const ColVariant *v = col_variant(ilog2(n), default_col_e(n), w);
     return v && p->nx % v->w == 0 && cols_wadj_available(*v) ? v : nullptr;
 }
 
@@ -214,6 +214,13 @@ int setup_row_axis(fft_plan_s *p, AxisPlan &ax, int n, const Schedule &sc) {
     ax.n = n;
     if (n == 1) return FFT_OK;
     int e = default_row_e(n);
+    // 512- and 1024-point rows: E = 32 makes them two stages with one exchange
+    // (64 x 512^2 rows 0.055 -> 0.049 ms, 16 x 1024^2 0.0555 -> 0.0535), where
+    // there are rows enough for its fewer threads and nothing asks for E = 16
+    // (the column pre-split's kernels and the one-launch small transforms)
+    if ((n == 512 || n == 1024) && (long long)p->nx * p->ny * p->batch >= 1 << 22 &&
+        !(p->nx > 1 && p->ny > 1 && (sc.split == 2 || small2d_available(p->nx, p->ny, p->batch, 16))))
+        e = 32;
     if (p->prec == FFT_PREC_SPLIT_FP16_TC) {
         if (!tc_rows_available(n)) return FFT_ERR_UNSUPPORTED;
         e = 16;
@@ -236,7 +243,6 @@ int setup_row_axis(fft_plan_s *p, AxisPlan &ax, int n, const Schedule &sc) {
         cudaFuncSetAttribute(ax.row->fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ax.row->smem);
     p->row_persist = sc.row_persist;
     p->row_pf = sc.row_pf;
-    p->col_pf = sc.col_pf;
     // long rows may go through the TMA landing-ring kernel (same E = 16
     // schedule and twiddle table as the plain row kernel)
     p->ring = sc.ring && ring_rows_available(n) && ax.row->e == 16 && p->prec == FFT_PREC_FP32;
@@ -325,7 +331,9 @@ int setup_col_axis(fft_plan_s *p, AxisPlan &ax, int n, int nx, long long tiles_p
     // small arrays: narrower tiles (down to 32-byte tile rows) until there is
     // a tile per SM (1024^2: 0.0144 -> 0.0120 ms; 512^2: 0.0105 -> 0.0084)
     while (w > 4 && tiles_per_w / w < p->num_sms && col_variant(ilog2(n), preferred_col_e(n, w / 2), w / 2)) w /= 2;
-    int e = preferred_col_e(n, w);
+    // still too few tiles to fill the SMs: the latency of one tile counts, and
+    // E = 16 has more threads on it (2048 x 512: 0.0146 -> 0.0130 ms)
+    int e = tiles_per_w / w < p->num_sms && n < 4096 ? default_col_e(n) : preferred_col_e(n, w);
     if (sc.col_kind == kColTile && sc.col_e > 0 && col_variant(ilog2(n), sc.col_e, w)) e = sc.col_e;
     if (sc.col_kind == kColTile && sc.col_w >= 2 && sc.col_w <= nx && col_variant(ilog2(n), e, sc.col_w)) w = sc.col_w;
     ax.col = col_variant(ilog2(n), e, w);
@@ -340,6 +348,7 @@ int setup_col_axis(fft_plan_s *p, AxisPlan &ax, int n, int nx, long long tiles_p
     if (grid > ntiles) grid = ntiles;
     if (grid < 1) grid = 1;
     ax.grid = (int)grid;
+    ax.pf = sc.col_pf >= 0 ? sc.col_pf : default_col_pf(n, ntiles / grid);
     int pt = 0, pg = 0;
     const ColVariant *sv = sc.col_stream ? stream_col_variant(n, nx, &pt, &pg, sc.col_tstore) : nullptr;
     if (sv && sv->w == ax.col->w && sv->box_rows == ax.col->box_rows) {
@@ -366,9 +375,12 @@ int setup_fourstep(fft_plan_s *p, int n) {
     const int L = ilog2(n);
     FourStepPlan &fs = p->fs;
     fs.n = n;
-    // n2 = 2^ceil(L/2), except that a length-8192 row (16-byte store chunks)
-    // is avoided while n1 stays <= 8192 (2^25: 8192 x 4096 measured faster)
-    fs.n2 = 1 << ((L + 1) / 2);
+    // n2 = 2^ceil(L/2), except where another split has the faster passes (2^24
+    // points in all, columns + rows): 2^17 and 2^18 with 256-point rows (0.099
+    // against 0.106 ms, 0.102 against 0.107), 2^21 and 2^22 with 4096-point ones
+    // (0.125 against 0.128, 0.129 against 0.144); and a length-8192 row (16-byte
+    // store chunks) is avoided while n1 stays <= 8192
+    fs.n2 = L == 17 || L == 18 ? 256 : L == 21 || L == 22 ? 4096 : 1 << ((L + 1) / 2);
     if (fs.n2 == 8192 && n / 4096 <= 8192) fs.n2 = 4096;
     // GB300FFT_FS_N2 / _FS_WA / _FS_EA / _FS_EB / _FS_WB: schedule
     // experiments (row length, tile width and elements per thread of pass A,
@@ -387,15 +399,28 @@ int setup_fourstep(fft_plan_s *p, int n) {
         fs.n2 = n / 4096;
         fs.m = fs.n2 / 4096;
     }
-    // pass A tile width: 4 from 2048 up, 8 at 1024, 16 below (measured; the
-    // 2D column pass's rule gives 8 at 2048, 0.31 vs 0.26 ms here)
-    int wa = fs.n1 >= 8192 ? 2 : fs.n1 >= 2048 ? 4 : fs.n1 == 1024 ? 8 : 16;
+    // pass A tile width: the 2D column pass's; narrower, down to 32-byte tile
+    // rows, until there is a tile per SM (not at 128 points: 4 x 2^14 points
+    // 0.0072 -> 0.0077 ms by it)
+    int wa = default_col_w(fs.n1, fs.n2);
+    while (wa > 4 && fs.n1 >= 256 && (long long)p->batch * (fs.n2 / wa) < p->num_sms &&
+           col_variant(ilog2(fs.n1), preferred_col_e(fs.n1, wa / 2), wa / 2))
+        wa /= 2;
     if (const char *ev = getenv("GB300FFT_FS_WA"))
         if (col_variant(ilog2(fs.n1), default_col_e(fs.n1), atoi(ev)) && atoi(ev) <= fs.n2) wa = atoi(ev);
     // E = 32 for the length-8192 column pass (measured 0.62 -> 0.52 ms at 2^26)
     const int rown = fs.n2 / fs.m;  // length of pass B's rows
-    int ea = fs.n1 == 8192 ? 32 : preferred_col_e(fs.n1, wa), eb = fourstep_row_e(rown);
+    // E = 16 as in setup_col_axis, and at 2048 points also while the last of a
+    // few rounds of one-per-SM tiles would be half empty (2^23 points, 512 such
+    // tiles: 0.0771 against 0.0756 ms; twice as many: 0.1385 against 0.1426)
+    const long long tiles_a = (long long)p->batch * (fs.n2 / wa);
+    const bool few = fs.n1 < 4096 && tiles_a < (fs.n1 == 2048 ? 4 : 1) * (long long)p->num_sms;
+    if (few && fs.n1 == 2048) wa = 4;
+    int ea = fs.n1 == 8192 ? 32 : few ? default_col_e(fs.n1) : preferred_col_e(fs.n1, wa), eb = fourstep_row_e(rown);
     int wb = fourstep_row_w(rown);
+    while (wb > 4 && rown >= 256 && (long long)p->batch * fs.m * (fs.n1 / wb) < p->num_sms &&
+           fourstep_row_variant(ilog2(rown), eb, wb / 2))
+        wb /= 2;
     if (const char *ev = getenv("GB300FFT_FS_EA"))
         if (col_variant(ilog2(fs.n1), atoi(ev), wa)) ea = atoi(ev);
     if (fs.m == 1) {
@@ -622,7 +647,9 @@ int setup_any_axis(fft_plan_s *p, AnyAxis &ax, int n, long long rows, int cols_n
     const bool fused = !(ev && atoi(ev) == 0);
     if (fused && !e1) ax.half = blu_half_variant(ax.M);
     if (!ax.half) {
-        ax.sub = create_dense(ax.M, 1, (int)rows, FFT_FORWARD, FFT_PREC_FP32, default_schedule(ax.M, 1), &rc);
+        Schedule ss = default_schedule(ax.M, 1);
+        if (const BluVariant *bv = blu_variant(ax.M)) ss.row_e = bv->e;  // the fused kernels share its twiddle table
+        ax.sub = create_dense(ax.M, 1, (int)rows, FFT_FORWARD, FFT_PREC_FP32, ss, &rc);
         if (!ax.sub) return rc;
     }
     for (int d = 0; d < 2; ++d) {
@@ -848,7 +875,8 @@ int run_fourstep(fft_plan_s *p, const float2 *src, float2 *dst, bool inv, cudaSt
         fs.map_base = src;
     }
     if (p->ev[0] && pass_event(p, 0, s) != cudaSuccess) return FFT_ERR_CUDA;
-    if (launch_cols(*fs.a, fs.map, fs.work, fs.tw_a, fs.n2, p->batch, 1, inv ? 2 : 0, p->status, fs.grid_a, 0, s) !=
+    if (launch_cols(*fs.a, fs.map, fs.work, fs.tw_a, fs.n2, p->batch, 1, inv ? 2 : 0, p->status, fs.grid_a,
+                    default_col_pf(fs.n1, (long long)p->batch * (fs.n2 / fs.a->w) / fs.grid_a), s) !=
         cudaSuccess)
         return FFT_ERR_CUDA;
     if (p->ev[1] && pass_event(p, 1, s) != cudaSuccess) return FFT_ERR_CUDA;
@@ -880,7 +908,7 @@ int run_columns(fft_plan_s *p, const float2 *src, float2 *dst, bool inv, cudaStr
     }
     if (p->ev[0] && pass_event(p, 0, s) != cudaSuccess) return FFT_ERR_CUDA;
     if (p->ev[1] && pass_event(p, 1, s) != cudaSuccess) return FFT_ERR_CUDA;
-    if (launch_cols(*cp.col, cp.map, dst, cp.tw, p->nx, p->batch, 1, inv ? 3 : 0, p->status, cp.grid, p->col_pf, s) !=
+    if (launch_cols(*cp.col, cp.map, dst, cp.tw, p->nx, p->batch, 1, inv ? 3 : 0, p->status, cp.grid, cp.pf, s) !=
         cudaSuccess)
         return FFT_ERR_CUDA;
     if (p->ev[2] && pass_event(p, 2, s) != cudaSuccess) return FFT_ERR_CUDA;
@@ -1025,7 +1053,7 @@ int run_dense(fft_plan_s *p, const void *in, void *out, int sign, const float *w
                                     p->batch, P,
                                     inv ? 1 : 0, p->status, cp.stream_grid, planar ? 1 : 0, s)
                : launch_cols(*cp.col, cp.map, dst, cp.tw, p->nx, p->batch, P, inv ? 1 : 0, p->status, cp.grid,
-                             p->col_pf, s);
+                             cp.pf, s);
     if (ec != cudaSuccess) return FFT_ERR_CUDA;
     if (p->ev[2] && pass_event(p, 2, s) != cudaSuccess) return FFT_ERR_CUDA;
     return FFT_OK;
@@ -1115,7 +1143,6 @@ fft_plan_t fft_plan_create_columns(int nx, int ny, int batch, int dir, int preci
     sc.col_stream = 0;  // the streaming pass needs rows stored in its own order
     sc.col_kind = kColTile;
     p->sched = sc;
-    p->col_pf = sc.col_pf;
     int rc = FFT_OK;
     if (cudaGetDevice(&p->device) != cudaSuccess ||
         cudaDeviceGetAttribute(&p->num_sms, cudaDevAttrMultiProcessorCount, p->device) != cudaSuccess)
@@ -1328,7 +1355,7 @@ int fft_weighted_power_adjoint(fft_plan_t p, const void *x, const void *w, void 
     int grid = p->num_sms * cols_wadj_ctas_per_sm(*v);
     if (grid > tiles) grid = (int)tiles;
     if (launch_cols_wadj(*v, p->wadj_map, yd, p->wadj_tw, static_cast<const float *>(w), static_cast<float *>(partials),
-                         p->nx, p->batch, p->status, grid, p->col_pf, s) != cudaSuccess)
+                         p->nx, p->batch, p->status, grid, p->sched.col_pf > 0 ? p->sched.col_pf : 0, s) != cudaSuccess)
         return FFT_ERR_CUDA;
     return FFT_OK;
 }
