@@ -141,13 +141,19 @@ __global__ void __launch_bounds__(ColShape<N, E, W>::THREADS, ColShape<N, E, W>:
 
 // Differentiation form, column half (P = 1).  For L = sum w |F x|^2 the
 // gradient is 2 F^H (w (.) X) with X = F x, and F^H = F_rows^H F_cols^H.
-// Each tile: the forward column transform, its outputs X written back into
-// the tile in natural order; one sweep over the tile that adds the tile's
-// loss partial sum of w |X|^2 (float, one per tile) and replaces X by
-// conj(w (.) X); the same forward engine over that, whose conjugated outputs
-// are F_cols^H (w (.) X), stored in place of the tile's input.  X itself
-// never reaches HBM: the pass reads the row pass's output and w and writes
-// the adjoint's column half.
+// Each tile: the forward column transform, whose outputs X stay in registers,
+// where they already are the next transform's inputs (a thread's outputs and
+// its inputs are both the elements tt + k * T); the tile's loss partial sum of
+// w |X|^2 (float, one per tile) and conj(w (.) X); the same forward engine over
+// that, whose conjugated outputs are F_cols^H (w (.) X), stored in place of the
+// tile's input.  X itself never reaches HBM: the pass reads the row pass's
+// output and w and writes the adjoint's column half.  Bound by the latency of
+// its exchanges and loads at 8 to 16 warps an SM; writing X back to the tile,
+// sweeping it and loading it again took 16 x 1024^2 (E = 16, with the row pass)
+// 0.182 ms, this 0.141; 64 x 512^2 0.172 -> 0.124, 8 x 2048^2 0.372 -> 0.323,
+// 256-point columns 0.143 -> 0.124.  The sweep remains at 2048 points with E =
+// 16 (64 registers: X and a three-stage engine spill), the faster form for few
+// tiles.
 template <int N, int E, int W>
 __global__ void __launch_bounds__(ColShape<N, E, W>::THREADS, ColShape<N, E, W>::MINB)
     k_cols_wadj(const __grid_constant__ CUtensorMap map, float2 *out, const float2 *__restrict__ tw,
@@ -157,6 +163,7 @@ __global__ void __launch_bounds__(ColShape<N, E, W>::THREADS, ColShape<N, E, W>:
     constexpr int R0 = Eng::R0;
     constexpr int T = Sh::T;
     constexpr int WARPS = Sh::THREADS / 32;
+    constexpr bool IN_REGS = N < 2048 || E >= 32;
     extern __shared__ __align__(128) unsigned char raw[];
     float2 *tile = reinterpret_cast<float2 *>(raw);
     uint64_t *bar = reinterpret_cast<uint64_t *>(raw + Sh::BAR_OFF);
@@ -220,23 +227,45 @@ __global__ void __launch_bounds__(ColShape<N, E, W>::THREADS, ColShape<N, E, W>:
 
         float part = 0.f;
         float2 v[E];
-        load_v(v);
-        auto all_read = [] { __syncthreads(); };
-        auto fwd_store = [&](int i, int cc, float2 x) { tile[i * W + cc] = x; };
-        Eng::template run<FftPolicy, true>(v, tile, tw, tt, c, SyncBlock{}, all_read, fwd_store);
-        __syncthreads();  // X complete in the tile, natural order
-        // w (.) X, its power and the conjugate, element by element: each row
-        // of W adjacent w values is one coalesced run (offsets < N * nx)
+        if constexpr (!IN_REGS) {
+            load_v(v);
+            auto all_read = [] { __syncthreads(); };
+            auto fwd_store = [&](int i, int cc, float2 x) { tile[i * W + cc] = x; };
+            Eng::template run<FftPolicy, true>(v, tile, tw, tt, c, SyncBlock{}, all_read, fwd_store);
+            __syncthreads();  // X complete in the tile, natural order
+            // w (.) X, its power and the conjugate, element by element: each row
+            // of W adjacent w values is one coalesced run (offsets < N * nx)
 #pragma unroll 4
-        for (int k = t; k < N * W; k += Sh::THREADS) {
-            const int i = k / W, cc = k % W;
-            const float wv = __ldg(wt + (i * nx + cc));
-            const float2 x = tile[k];
-            part = fmaf(wv, fmaf(x.x, x.x, x.y * x.y), part);
-            tile[k] = make_float2(wv * x.x, -(wv * x.y));
+            for (int k = t; k < N * W; k += Sh::THREADS) {
+                const int i = k / W, cc = k % W;
+                const float wv = __ldg(wt + (i * nx + cc));
+                const float2 x = tile[k];
+                part = fmaf(wv, fmaf(x.x, x.x, x.y * x.y), part);
+                tile[k] = make_float2(wv * x.x, -(wv * x.y));
+            }
+            __syncthreads();  // conj(w (.) X) complete in the tile
+            load_v(v);
+        } else {
+            // this tile's w into L2 while the first transform runs
+#pragma unroll 1
+            for (int i = t; i < N; i += Sh::THREADS) asm volatile("prefetch.global.L2 [%0];" ::"l"(wt + i * nx));
+            load_v(v);
+            float2 x[E];
+            int m = 0;
+            auto keep = [&](int, int, float2 y) { x[m++] = y; };  // X at tt + m * T
+            Eng::template run<FftPolicy, true>(v, tile, tw, tt, c, SyncBlock{}, [] {}, keep);
+            // w (.) X, its power and the conjugate: X at tt + k * T, k = bb + r *
+            // (E / R0), is the next transform's input (bb, r)
+#pragma unroll
+            for (int bb = 0; bb < E / R0; ++bb)
+#pragma unroll
+                for (int r = 0; r < R0; ++r) {
+                    const int k = bb + r * (E / R0);
+                    const float wv = __ldg(wt + ((tt + k * T) * nx + c));
+                    part = fmaf(wv, fmaf(x[k].x, x[k].x, x[k].y * x[k].y), part);
+                    v[bb * R0 + r] = make_float2(wv * x[k].x, -(wv * x[k].y));
+                }
         }
-        __syncthreads();  // conj(w (.) X) complete in the tile
-        load_v(v);
         auto after_reads = [&] {
             __syncthreads();
             if (t == 0 && next < ntiles) {
@@ -333,7 +362,9 @@ void reg_col(int eslot) {
     en.v.box_rows = Sh::BOXR;
     en.v.tw_size = Sched<N, E>::tw_size;
     en.movemap = (const void *)k_cols_movemap<N, E, W>;
-    if constexpr (N >= 32 && N <= 2048 && E <= 16 && THREADS_OK<N, E, W>::value) en.wadj = (const void *)k_cols_wadj<N, E, W>;
+    // the shapes the plan chooses from
+    constexpr bool WADJ = N >= 32 && (N <= 256 ? E == 16 : N <= 1024 ? E == 32 : N == 2048 && (E == 64 ? W == 8 : W <= 4));
+    if constexpr (WADJ && THREADS_OK<N, E, W>::value) en.wadj = (const void *)k_cols_wadj<N, E, W>;
 }
 
 template <int N, int E>

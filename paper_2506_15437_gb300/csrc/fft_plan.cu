@@ -59,9 +59,8 @@ bool is_pow2(long long n) { return n >= 1 && (n & (n - 1)) == 0; }
 // pass runs without a pre-split and has a compiled fused variant.
 // Its tiles are the widest of at most 64 KiB (whole warps, W adjacent
 // columns), not the narrowed tiles small plans use for their column pass:
-// two CTAs per SM, one transforming while the other loads (measured against
-// the column pass's own 128 KiB tiles: 8 x 2048^2 step 0.495 -> 0.483 ms,
-// 32 x 1024^2 0.461 -> 0.452).
+// two CTAs per SM, one transforming while the other loads (16 x 1024^2, with the
+// row pass: 8 columns 0.141 ms, 16 columns 0.144, 4 columns 0.150).
 const ColVariant *wadj_variant(fft_plan_s *p) {
     if (!p || p->kind != 0 || p->prec != FFT_PREC_FP32 || p->dir != FFT_FORWARD) return nullptr;
     if (p->any || p->fs.n1 > 0 || p->axes == 2 || p->rows.n < 2 || !p->rows.row || !p->cols.col) return nullptr;
@@ -70,9 +69,17 @@ const ColVariant *wadj_variant(fft_plan_s *p) {
     // 2 x 4096^2 step slower than the unfused one
     const int n = p->ny;
     if (n > 2048 || !is_pow2(n)) return nullptr;
-    int w = default_col_w(n, p->nx);
-    while (w > 2 && (long long)n * w * sizeof(float2) > 65536) w >>= 1;
-    const ColVariant *v = col_variant(ilog2(n), default_col_e(n), w);
+    int w = default_col_w(n, p->nx), e = n == 512 || n == 1024 ? 32 : default_col_e(n);
+    if (n == 2048) {
+        // 128 KiB tiles with one exchange per transform (E = 64), one to an SM,
+        // where the SMs have eight each or more (8 x 2048^2 0.372 -> 0.323 ms
+        // against 64 KiB tiles with E = 16); with fewer the last round's idle
+        // SMs cost more than that gains (2 x 2048^2 0.104 against 0.110)
+        const bool many = p->nx >= 8 && (long long)(p->nx / 8) * p->batch >= 8LL * p->num_sms;
+        e = many ? 64 : 16;
+        w = many ? 8 : w > 4 ? 4 : w;
+    }
+    const ColVariant *v = col_variant(ilog2(n), e, w);
     return v && p->nx % v->w == 0 && cols_wadj_available(*v) ? v : nullptr;
 }
 
