@@ -222,10 +222,11 @@ int setup_row_axis(fft_plan_s *p, AxisPlan &ax, int n, const Schedule &sc) {
     if (n == 1) return FFT_OK;
     int e = default_row_e(n);
     // 512- and 1024-point rows: E = 32 makes them two stages with one exchange
-    // (64 x 512^2 rows 0.055 -> 0.049 ms, 16 x 1024^2 0.0555 -> 0.0535), where
-    // there are rows enough for its fewer threads and nothing asks for E = 16
-    // (the column pre-split's kernels and the one-launch small transforms)
-    if ((n == 512 || n == 1024) && (long long)p->nx * p->ny * p->batch >= 1 << 22 &&
+    // (2^24 points: 0.0433 -> 0.0422 ms and 0.0440 -> 0.0430; 2^21 points of 1024
+    // 0.0080 -> 0.0068), where there are rows enough for its fewer threads and
+    // nothing asks for E = 16 (the column pre-split's kernels and the one-launch
+    // small transforms)
+    if ((n == 512 || n == 1024) && (long long)p->nx * p->ny * p->batch >= 1 << 20 &&
         !(p->nx > 1 && p->ny > 1 && (sc.split == 2 || small2d_available(p->nx, p->ny, p->batch, 16))))
         e = 32;
     if (p->prec == FFT_PREC_SPLIT_FP16_TC) {

@@ -21,15 +21,25 @@ namespace gb300fft {
 #define ROWMINB32 2  // 256-thread CTAs with E = 32: two per SM (128 registers)
 #endif
 
+// Rows per CTA: as few as make 64 threads (the pass is bound by the latency of
+// its loads and exchanges, and a barrier over 256 threads holds up rows that
+// have nothing to do with each other).  2^24 points, 256-thread CTAs against
+// these: 128 points 0.0453 -> 0.0432 ms, 512 (E = 16) 0.0504 -> 0.0433, 1024
+// (E = 16) 0.0517 -> 0.0440, 2^25 points of 2048 0.0977 -> 0.0872; 1024 points
+// with E = 32 0.0515 -> 0.0430, 6.2 TB/s.
 template <int N, int E>
 struct RowShape {
     static constexpr int T = N / E;
-    static constexpr int ROWS = (T >= 256) ? 1 : 256 / T;
+    static constexpr int CTA = E == 16 || (E == 32 && N >= 512) ? 64 : 256;
+    static constexpr int ROWS = (T >= CTA) ? 1 : CTA / T;
     static constexpr int THREADS = ROWS * T;
-    // resident CTAs the register budget must allow: 64 registers per thread
-    // for 512-thread CTAs with E <= 16, at most 85 for 256-thread ones
+    // resident CTAs the register budget must allow: with E <= 16 64 registers
+    // per thread for 512-thread CTAs, at most 85 for smaller ones; 128 with
+    // E = 32
     static constexpr int MINB = THREADS >= 512 ? (E >= 32 ? 512 : 1024) / THREADS
-                                               : (THREADS >= 256 ? (E < 32 ? 3 : ROWMINB32) : 1);
+                                : E == 32 && N >= 512 ? 512 / THREADS
+                                : THREADS >= 256 ? (E < 32 ? 3 : ROWMINB32)
+                                : E == 16 ? 768 / THREADS : 1;
     using Eng = Engine<N, E, 1, PadShift<E>::value, RowPadShift1<E>::value>;
     static constexpr size_t SMEM = sizeof(float2) * (size_t)ROWS * Eng::SMEM_ELEMS;
 };

@@ -54,7 +54,7 @@ def test_short_columns_with_tiles_to_spare(g, ny, batch):
 @pytest.mark.parametrize("nx", [512, 1024])
 @pytest.mark.parametrize("below", [0, 1])
 def test_rows(g, nx, below):
-    _check(g, nx, 1, (1 << 22) // nx - below)
+    _check(g, nx, 1, (1 << 20) // nx - below)
 
 
 @pytest.mark.parametrize("log2n", range(14, 25))
