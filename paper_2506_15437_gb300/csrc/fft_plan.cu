@@ -225,8 +225,11 @@ int setup_row_axis(fft_plan_s *p, AxisPlan &ax, int n, const Schedule &sc) {
     // (2^24 points: 0.0433 -> 0.0422 ms and 0.0440 -> 0.0430; 2^21 points of 1024
     // 0.0080 -> 0.0068), where there are rows enough for its fewer threads and
     // nothing asks for E = 16 (the column pre-split's kernels and the one-launch
-    // small transforms)
-    if ((n == 512 || n == 1024) && (long long)p->nx * p->ny * p->batch >= 1 << 20 &&
+    // small transforms).  4096-point rows have three stages either way; their
+    // 128-thread CTAs win once there are rows for several rounds of them (2^25
+    // points 0.0957 -> 0.0945 ms, 2^26 0.184 -> 0.181; 2^22 points 0.0136 ->
+    // 0.0145, so not there).
+    if ((long long)p->nx * p->ny * p->batch >= (n == 4096 ? 1 << 24 : 1 << 20) && (n == 512 || n == 1024 || n == 4096) &&
         !(p->nx > 1 && p->ny > 1 && (sc.split == 2 || small2d_available(p->nx, p->ny, p->batch, 16))))
         e = 32;
     if (p->prec == FFT_PREC_SPLIT_FP16_TC) {

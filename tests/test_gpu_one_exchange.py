@@ -1,4 +1,4 @@
-"""Columns, rows and four-step passes of 512 to 2048 points with 32 and 64 elements per thread (GPU).
+"""Columns, rows and four-step passes of 512 to 4096 points with 32 and 64 elements per thread (GPU).
 
 Each length sits on both sides of the rules that choose them (enough tiles for
 the SMs, enough points for the rows), with the narrowest and widest tiles,
@@ -51,10 +51,10 @@ def test_short_columns_with_tiles_to_spare(g, ny, batch):
     _check(g, 1024, ny, batch)
 
 
-@pytest.mark.parametrize("nx", [512, 1024])
+@pytest.mark.parametrize("nx,points", [(512, 1 << 20), (1024, 1 << 20), (4096, 1 << 24)])
 @pytest.mark.parametrize("below", [0, 1])
-def test_rows(g, nx, below):
-    _check(g, nx, 1, (1 << 20) // nx - below)
+def test_rows(g, nx, points, below):
+    _check(g, nx, 1, points // nx - below)
 
 
 @pytest.mark.parametrize("log2n", range(14, 25))
