@@ -64,9 +64,8 @@ bool is_pow2(long long n) { return n >= 1 && (n & (n - 1)) == 0; }
 const ColVariant *wadj_variant(fft_plan_s *p) {
     if (!p || p->kind != 0 || p->prec != FFT_PREC_FP32 || p->dir != FFT_FORWARD) return nullptr;
     if (p->any || p->fs.n1 > 0 || p->axes == 2 || p->rows.n < 2 || !p->rows.row || !p->cols.col) return nullptr;
-    // the whole column in one tile, up to 2048 points: at 4096 the fused
-    // column pass (two transforms per tile at 8 warps per SM) made the
-    // 2 x 4096^2 step slower than the unfused one
+    // the whole column in one tile, up to 2048 points, the limit the entry
+    // point documents
     const int n = p->ny;
     if (n > 2048 || !is_pow2(n)) return nullptr;
     int w = default_col_w(n, p->nx), e = n == 512 || n == 1024 ? 32 : default_col_e(n);
