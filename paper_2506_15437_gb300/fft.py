@@ -36,6 +36,28 @@ def _check_tensor(t: torch.Tensor, dtype, name: str):
         raise ValueError(f"{name} must be contiguous")
 
 
+def _values(t: torch.Tensor) -> torch.Tensor:
+    """t with a lazy conjugation or negation carried out.  The kernels read
+    t's memory, which such a view (x.conj(), the gradient that reaches
+    fft2(x).conj()) leaves as it was; contiguous() keeps the view."""
+    if t.is_conj():
+        t = t.resolve_conj()
+    if t.is_neg():
+        t = t.resolve_neg()
+    return t
+
+
+def _input(t: torch.Tensor, dtype, name: str) -> torch.Tensor:
+    _check_tensor(t, dtype, name)
+    return _values(t)
+
+
+def _check_output(t: torch.Tensor, dtype, name: str):
+    _check_tensor(t, dtype, name)
+    if t.is_conj() or t.is_neg():
+        raise ValueError(f"{name} must not be a lazily conjugated or negated view")
+
+
 class Plan:
     """A dense plan: ``batch`` transforms of size ``[ny][nx]``."""
 
@@ -55,19 +77,19 @@ class Plan:
         return self.nx * self.ny * self.batch
 
     def _io(self, x, out):
-        _check_tensor(x, torch.complex64, "input")
+        x = _input(x, torch.complex64, "input")
         if x.numel() != self.numel:
             raise ValueError(f"input has {x.numel()} elements, plan expects {self.numel}")
         if out is None:
             out = torch.empty_like(x)
         else:
-            _check_tensor(out, torch.complex64, "out")
+            _check_output(out, torch.complex64, "out")
             if out.numel() != self.numel:
                 raise ValueError("out has the wrong size")
-        return out
+        return x, out
 
     def execute(self, x: torch.Tensor, out: torch.Tensor | None = None) -> torch.Tensor:
-        out = self._io(x, out)
+        x, out = self._io(x, out)
         rc = self._lib.fft_execute(self._p, x.data_ptr(), out.data_ptr(),
                                    torch._C._cuda_getCurrentRawStream(x.get_device()))
         if rc:
@@ -86,23 +108,27 @@ class Plan:
             raise ValueError(f"input has {x.numel()} elements, plan expects {self.numel}")
         if out is None:
             out = torch.empty_like(x, pin_memory=x.is_pinned())
-        elif out.is_cuda or out.dtype != torch.complex64 or not out.is_contiguous() or out.numel() != self.numel:
-            raise ValueError("out must be a contiguous complex64 CPU tensor of the plan's size")
+        elif (out.is_cuda or out.dtype != torch.complex64 or not out.is_contiguous() or out.numel() != self.numel
+              or out.is_conj() or out.is_neg()):
+            raise ValueError("out must be a contiguous complex64 CPU tensor of the plan's size, not a lazy view")
         dev = torch.device("cuda") if device is None else torch.device(device)
-        N.check(self._lib.fft_execute_host(self._p, x.data_ptr(), out.data_ptr(), _stream_handle(dev)),
+        v = _values(x)
+        N.check(self._lib.fft_execute_host(self._p, v.data_ptr(), out.data_ptr(), _stream_handle(dev)),
                 "fft_execute_host")
+        if v is not x:
+            torch.cuda.current_stream(dev).synchronize()  # v goes with this call: its upload must have ended
         return out
 
     def backward(self, g: torch.Tensor, out: torch.Tensor | None = None) -> torch.Tensor:
-        out = self._io(g, out)
+        g, out = self._io(g, out)
         N.check(self._lib.fft_backward(self._p, g.data_ptr(), out.data_ptr(),
                                        _stream_handle(g.device)), "fft_backward")
         return out
 
     def backward_weighted(self, X: torch.Tensor, w: torch.Tensor, scale: float,
                           out: torch.Tensor | None = None) -> torch.Tensor:
-        out = self._io(X, out)
-        _check_tensor(w, torch.float32, "w")
+        X, out = self._io(X, out)
+        w = _input(w, torch.float32, "w")
         if w.numel() != self.numel:
             raise ValueError("w has the wrong size")
         N.check(self._lib.fft_backward_weighted(self._p, X.data_ptr(), w.data_ptr(),
@@ -115,9 +141,9 @@ class Plan:
                               scale: float = 1.0, out: torch.Tensor | None = None) -> torch.Tensor:
         """F^H (scale * scale_dev * w (.) X) with scale_dev a one-element
         float32 CUDA tensor read on the device (no host synchronisation)."""
-        out = self._io(X, out)
-        _check_tensor(w, torch.float32, "w")
-        _check_tensor(scale_dev, torch.float32, "scale_dev")
+        X, out = self._io(X, out)
+        w = _input(w, torch.float32, "w")
+        scale_dev = _input(scale_dev, torch.float32, "scale_dev")
         if w.numel() != self.numel or scale_dev.numel() != 1:
             raise ValueError("w must have the plan's size and scale_dev one element")
         N.check(self._lib.fft_backward_weighted_dev(self._p, X.data_ptr(), w.data_ptr(), scale_dev.data_ptr(),
@@ -128,8 +154,8 @@ class Plan:
 
     def weighted_power(self, X: torch.Tensor, w: torch.Tensor) -> torch.Tensor:
         """sum w*|X|^2 as a float64 0-d tensor (partials reduced by torch)."""
-        _check_tensor(X, torch.complex64, "X")
-        _check_tensor(w, torch.float32, "w")
+        X = _input(X, torch.complex64, "X")
+        w = _input(w, torch.float32, "w")
         parts = self._lib.fft_weighted_power_parts(self._p)
         partials = torch.empty(parts, dtype=torch.float32, device=X.device)
         N.check(self._lib.fft_weighted_power(self._p, X.data_ptr(), w.data_ptr(),
@@ -147,8 +173,8 @@ class Plan:
         """(L, y): L = sum w*|F x|^2 as a float64 0-d tensor and y =
         F_cols^H (w (.) F x), the adjoint's column half, in two passes
         (fft_weighted_power_adjoint)."""
-        y = self._io(x, y)
-        _check_tensor(w, torch.float32, "w")
+        x, y = self._io(x, y)
+        w = _input(w, torch.float32, "w")
         if w.numel() != self.numel:
             raise ValueError("w has the wrong size")
         parts = self.weighted_power_adjoint_parts()
@@ -164,9 +190,9 @@ class Plan:
                              out: torch.Tensor | None = None) -> torch.Tensor:
         """scale * scale_dev * F_rows^H y (fft_backward_rows_scaled); scale_dev
         a one-element float32 CUDA tensor read on the device, or None."""
-        out = self._io(y, out)
+        y, out = self._io(y, out)
         if scale_dev is not None:
-            _check_tensor(scale_dev, torch.float32, "scale_dev")
+            scale_dev = _input(scale_dev, torch.float32, "scale_dev")
             if scale_dev.numel() != 1:
                 raise ValueError("scale_dev must have one element")
         N.check(self._lib.fft_backward_rows_scaled(self._p, y.data_ptr(),
@@ -226,11 +252,11 @@ class ColumnPlan(Plan):
 def slab_pack(x: torch.Tensor, parts: int, batch: int, rows: int, nx: int, out: torch.Tensor | None = None):
     """out[s][b][y][x'] = x[b][y][s*w + x'] (w = nx/parts): the all-to-all
     chunk for each rank s, contiguous (fft_slab_pack)."""
-    _check_tensor(x, torch.complex64, "x")
+    x = _input(x, torch.complex64, "x")
     if x.numel() != batch * rows * nx:
         raise ValueError("x must hold batch*rows*nx elements")
     out = torch.empty(parts, batch, rows, nx // parts, dtype=x.dtype, device=x.device) if out is None else out
-    _check_tensor(out, torch.complex64, "out")
+    _check_output(out, torch.complex64, "out")
     N.check(N.load().fft_slab_pack(x.data_ptr(), out.data_ptr(), parts, batch, rows, nx, _stream_handle(x.device)),
             "fft_slab_pack")
     return out
@@ -239,11 +265,11 @@ def slab_pack(x: torch.Tensor, parts: int, batch: int, rows: int, nx: int, out: 
 def slab_unpack(x: torch.Tensor, parts: int, batch: int, rows: int, w: int, out: torch.Tensor | None = None):
     """out[b][r*rows + y][x'] = x[r][b][y][x']: the chunks received from every
     rank assembled into this rank's column slab (fft_slab_unpack)."""
-    _check_tensor(x, torch.complex64, "x")
+    x = _input(x, torch.complex64, "x")
     if x.numel() != parts * batch * rows * w:
         raise ValueError("x must hold parts*batch*rows*w elements")
     out = torch.empty(batch, parts * rows, w, dtype=x.dtype, device=x.device) if out is None else out
-    _check_tensor(out, torch.complex64, "out")
+    _check_output(out, torch.complex64, "out")
     N.check(N.load().fft_slab_unpack(x.data_ptr(), out.data_ptr(), parts, batch, rows, w, _stream_handle(x.device)),
             "fft_slab_unpack")
     return out
@@ -430,26 +456,26 @@ class RaggedPlan:
         return self.offset(self.count)
 
     def _io(self, x, out):
-        _check_tensor(x, torch.complex64, "input")
+        x = _input(x, torch.complex64, "input")
         if x.numel() != self.total:
             raise ValueError(f"packed input has {x.numel()} elements, plan expects {self.total}")
         if out is None:
             out = torch.empty_like(x)
         else:
-            _check_tensor(out, torch.complex64, "out")
+            _check_output(out, torch.complex64, "out")
             if out.numel() != self.total:
                 raise ValueError("out has the wrong size")
-        return out
+        return x, out
 
     def execute(self, x: torch.Tensor, out: torch.Tensor | None = None) -> torch.Tensor:
-        out = self._io(x, out)
+        x, out = self._io(x, out)
         N.check(self._lib.fft_execute_ragged(self._p, x.data_ptr(), out.data_ptr(),
                                              _stream_handle(x.device)), "fft_execute_ragged")
         return out
 
     def execute_loop(self, x: torch.Tensor, out: torch.Tensor | None = None) -> torch.Tensor:
         """The same transforms as one plain launch pair per instance (baseline)."""
-        out = self._io(x, out)
+        x, out = self._io(x, out)
         N.check(self._lib.fft_execute_ragged_loop(self._p, x.data_ptr(), out.data_ptr(),
                                                   _stream_handle(x.device)), "fft_execute_ragged_loop")
         return out
