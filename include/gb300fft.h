@@ -372,15 +372,30 @@ int fft_plan_describe(fft_plan_t p, char *buf, int len);
  * `radices` (capacity 16) or a negative error. */
 int fft_debug_radices(int n, int axis, int *radices);
 
-/* The mixed-radix schedule of length n (2 <= n <= 2^24; Sections 6-7's
- * uneven sizes): for n = 2^a 3^b 5^c 7^d 11^e 13^f <= 14336 the stage radices of the
- * one-CTA kernel, first stage first, written to `radices` (capacity 16) and
- * their count returned, *n1 = *n2 = 0; for longer such n, 0 returned and the
+/* The mixed-radix factorisation of length n (2 <= n <= 2^24; Sections 6-7's
+ * uneven sizes): for n = 2^a 3^b 5^c 7^d 11^e 13^f <= 14336 one with the fewest
+ * stages the compiled radices allow, written to `radices` (capacity 16) and
+ * their count returned, *n1 = *n2 = 0 (the kernels run that many stages, of
+ * radices that depend on the launch too: fft_debug_mixed_launch; a single stage
+ * of 8 or more that is no prime runs as two); for longer such n, 0 returned and the
  * four-step split n = n1 * n2 written (columns of length n1, then rows of
  * length n2); FFT_ERR_INVALID_SIZE when n has a prime factor above 13 or is
  * out of range, FFT_ERR_INVALID_ARG for NULL pointers.  Host only: no
  * device call. */
 int fft_debug_mixed_plan(int n, int *radices, int *n1, int *n2);
+
+/* The launch a plan makes of one mixed-radix pass: `count` transforms of length
+ * n (13-smooth, 2 <= n <= 14336) in all, along contiguous rows (nx = 0) or down
+ * the columns of [n][nx] slices (nx > 0); fourstep != 0 for a pass of a
+ * four-step transform, with n1 > 0 for its second one (rows, n1 to a
+ * transform).  Writes to the host array info[24]: transforms per thread (1, or
+ * 2 side by side), transforms per CTA W, threads, shared-memory bytes, largest
+ * radix compiled into the kernel, skew (buffer elements left out after each
+ * block of the first digit), buffer elements per transform (pair), the stage
+ * count S, then the S stage radices, first stage first, and zeros.
+ * FFT_ERR_INVALID_SIZE for another n, FFT_ERR_INVALID_ARG for a NULL info, a
+ * negative nx or n1, both of them, or count < 1.  Host only: no device call. */
+int fft_debug_mixed_launch(int n, int nx, long long count, int fourstep, int n1, int *info);
 
 /*
  * fft_debug_row_variant -- launch shape of the compiled row-pass kernel for

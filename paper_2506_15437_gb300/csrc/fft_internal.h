@@ -356,8 +356,10 @@ constexpr int kMixedOneThreads = 1024;  // of 64 registers
 const void *mixed_one_fn(bool cols, bool fs);
 bool mixed_factor(int n, MixedStages *st);  // false unless n = 2^a 3^b 5^c 7^d 11^e 13^f <= kMixedMaxN
 cudaError_t build_mixed_twiddles(float2 *tw, const MixedStages &st, cudaStream_t s);
-// 0 on success; `count` transforms in all; fourstep: a pass of a four-step
-// transform, the second one (rows layout) with fs_n1 > 0 rows per transform
+// The launch for `count` transforms in all, 0 on success; fourstep: a pass of a
+// four-step transform, the second one (rows layout) with fs_n1 > 0 rows per
+// transform.  Host only; mixed_prepare also readies the kernel.
+int mixed_layout(const MixedStages &st, bool cols, int nx, long long count, MixedLaunch *out, bool fourstep, int fs_n1);
 int mixed_prepare(const MixedStages &st, bool cols, int nx, long long count, MixedLaunch *out, bool fourstep = false,
                   int fs_n1 = 0);
 // n = n1 n2 with both factors mixed-radix lengths (<= kMixedMaxN), n1 and

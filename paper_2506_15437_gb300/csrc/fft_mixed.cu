@@ -7,7 +7,8 @@
 // at plan time (15, 14, 12, 10, 9 and 6 are two-level DFTs in registers with
 // compile-time inner twiddles; the odd primes 3 .. 13 one symmetric-pair DFT
 // each): the fewest stages these radices allow, since each stage is one pass
-// through shared memory and one barrier.  One CTA owns whole transforms: the
+// through shared memory and one barrier (mixed_factor has the count,
+// pair_stages chooses the radices and their order).  One CTA owns whole transforms: the
 // first stage reads global memory, the last writes it.
 //
 // Two layouts: rows (transforms along contiguous rows, W rows per CTA) and
@@ -126,10 +127,12 @@ bool mixed_factor(int n, MixedStages *st) {
         while (rest % R == 0)
             if (!push(R)) return false;
     if (rest != 1) return false;
-    // the greedy schedule above is kept where no schedule has fewer stages
-    // (e.g. 3000 = 8 15 5 5); otherwise the first of the fewest, radices
+    // the greedy factorisation above is kept where none has fewer stages (e.g.
+    // 3000 = 8 15 5 5); otherwise the first of the fewest, radices
     // non-increasing (1000 = 10 10 10 in place of 8 5 5 5, 1728 = 16 12 9 in
-    // place of 16 4 9 3, 96 = 16 6 in place of 16 2 3)
+    // place of 16 4 9 3, 96 = 16 6 in place of 16 2 3).  The kernels run S
+    // stages, of pair_stages' radices; these ones enter mixed_layout's rule for
+    // small launches.
     for (int d = 1; d < S; ++d) {
         int r[kMixedMaxStages];
         if (factor_exact(n, d, 16, r)) {
@@ -326,8 +329,8 @@ int mixed_block(const MixedStages &m, int words, int rmax, size_t smem) {
 }
 }  // namespace
 
-int mixed_prepare(const MixedStages &st, bool cols, int nx, long long count, MixedLaunch *out, bool fourstep,
-                  int fs_n1) {
+int mixed_layout(const MixedStages &st, bool cols, int nx, long long count, MixedLaunch *out, bool fourstep,
+                 int fs_n1) {
     MixedLaunch L;
     L.cols = cols;
     L.nx = cols ? nx : 0;
@@ -363,9 +366,14 @@ int mixed_prepare(const MixedStages &st, bool cols, int nx, long long count, Mix
     // (single-stage rows: 2^20 of 7 points 0.024 ms with 64 threads, 0.036 with
     // 32; 2^21 of 3 points 0.024 and 0.019)
     L.T = S == 1 ? (st.n < 5 ? 32 : 64) : std::min(mixed_block(L.m, words, L.rmax, L.smem), L.T_most);
-    if (!smem_ok(mixed_fn(L.rmax, cols, fs), L.smem)) return -1;
     *out = L;
     return 0;
+}
+
+int mixed_prepare(const MixedStages &st, bool cols, int nx, long long count, MixedLaunch *out, bool fourstep,
+                  int fs_n1) {
+    if (mixed_layout(st, cols, nx, count, out, fourstep, fs_n1) != 0) return -1;
+    return smem_ok(mixed_fn(out->rmax, cols, out->fs.n1 > 0), out->smem) ? 0 : -1;
 }
 
 bool mixed_split(int n, int *n1, int *n2) {
@@ -412,6 +420,25 @@ cudaError_t launch_mixed(const MixedLaunch &L, const float2 *tw, const float2 *i
 }
 
 }  // namespace gb300fft
+
+// The launch a plan makes of one mixed-radix pass.
+extern "C" int fft_debug_mixed_launch(int n, int nx, long long count, int fourstep, int n1, int *info) {
+    if (!info || nx < 0 || count < 1 || n1 < 0 || (nx > 0 && n1 > 0)) return FFT_ERR_INVALID_ARG;
+    gb300fft::MixedStages st;
+    gb300fft::MixedLaunch L;
+    if (!gb300fft::mixed_factor(n, &st)) return FFT_ERR_INVALID_SIZE;
+    if (gb300fft::mixed_layout(st, nx > 0, nx, count, &L, fourstep != 0, n1) != 0) return FFT_ERR_UNSUPPORTED;
+    info[0] = L.rmax > 0 ? 2 : 1;
+    info[1] = L.W;
+    info[2] = L.T;
+    info[3] = (int)L.smem;
+    info[4] = L.rmax > 0 ? L.rmax : 16;
+    info[5] = L.m.skew;
+    info[6] = L.m.buf_elems;
+    info[7] = L.m.S;
+    for (int k = 0; k < 16; ++k) info[8 + k] = k < L.m.S ? L.m.radix[k] : 0;
+    return FFT_OK;
+}
 
 // The float constants the composite-radix DFTs multiply by, as the
 // compiler evaluates them (host copy of the same constexpr functions).
