@@ -362,7 +362,9 @@ int fft_plan_autotune(fft_plan_t p, void *stream);
  * fft_plan_describe -- the schedule a plan runs, as a NUL-terminated JSON
  * object written to the host buffer `buf` of `len` bytes: kernel names,
  * elements per thread, tile widths, column pre-split, grids and stage radices
- * of each pass.  Returns the number of characters needed (excluding the NUL);
+ * of each pass.  Plans that go axis by axis name each axis's method: mixed
+ * radix, its four-step split, or the Bluestein form that runs ("form").
+ * Returns the number of characters needed (excluding the NUL);
  * the output is truncated when that is >= len.
  */
 int fft_plan_describe(fft_plan_t p, char *buf, int len);

@@ -1543,20 +1543,23 @@ int fft_plan_describe(fft_plan_t p, char *buf, int len) {
         k = snprintf(tmp, sizeof tmp, "{\"kind\": \"ragged\", \"kernel\": \"k_ragged\"}");
     } else if (p->any) {
         const gb300fft::AnyPlan &ap = *p->any;
-        // "fused": the length-M Bluestein form of this padded length (0 five
-        // passes, 1 two, 2 one); "half_q" > 0: the one-pass form over
-        // transforms of that length runs in its place
-        auto fused = [](const gb300fft::AnyAxis &ax) {
-            return ax.half ? (ax.M > 8192 ? 0 : ax.M > 2048 ? 1 : 2) : ax.fused ? (ax.fused_one ? 2 : 1) : 0;
+        // "form": the Bluestein form that runs ("" for an axis without one);
+        // "fused": the length-M form of this padded length (0 five passes, 1
+        // two, 2 one), which does not run where "half_q" > 0, the length of the
+        // one-pass form's transforms
+        auto axis = [](const gb300fft::AnyAxis &ax, char *o, int cap) {
+            const int fused = ax.half ? (ax.M > 8192 ? 0 : ax.M > 2048 ? 1 : 2) : ax.fused ? (ax.fused_one ? 2 : 1) : 0;
+            const char *form = !ax.M ? "" : ax.half ? "half" : fused == 2 ? "one_pass" : fused == 1 ? "two_pass" : "five_pass";
+            snprintf(o, cap,
+                     "{\"n\": %d, \"bluestein_m\": %d, \"form\": \"%s\", \"fused\": %d, \"half_q\": %d, \"mixed\": %d, "
+                     "\"mixed_fourstep\": [%d, %d]}",
+                     ax.n, ax.M, form, fused, ax.half ? ax.half->q : 0, ax.mixed ? 1 : 0, ax.n1, ax.n2);
         };
-        auto half = [](const gb300fft::AnyAxis &ax) { return ax.half ? ax.half->q : 0; };
+        char x[256], y[256];
+        axis(ap.x, x, sizeof x);
+        axis(ap.y, y, sizeof y);
         k = snprintf(tmp, sizeof tmp,
-                     "{\"kind\": \"any\", \"precision\": \"fp32\", \"x\": {\"n\": %d, \"bluestein_m\": %d, "
-                     "\"fused\": %d, \"half_q\": %d, \"mixed\": %d, \"mixed_fourstep\": [%d, %d]}, \"y\": {\"n\": %d, "
-                     "\"bluestein_m\": %d, \"fused\": %d, \"half_q\": %d, \"mixed\": %d, \"mixed_fourstep\": [%d, %d]}, "
-                     "\"transposes\": %d}",
-                     ap.x.n, ap.x.M, fused(ap.x), half(ap.x), ap.x.mixed ? 1 : 0, ap.x.n1, ap.x.n2,
-                     ap.y.n, ap.y.M, fused(ap.y), half(ap.y), ap.y.mixed ? 1 : 0, ap.y.n1, ap.y.n2,
+                     "{\"kind\": \"any\", \"precision\": \"fp32\", \"x\": %s, \"y\": %s, \"transposes\": %d}", x, y,
                      (p->nx > 1 && p->ny > 1 && !ap.y_cols) ? 2 : 0);
     } else if (p->fs.n1 > 0) {
         const gb300fft::FourStepPlan &fs = p->fs;
