@@ -1546,14 +1546,16 @@ int fft_plan_describe(fft_plan_t p, char *buf, int len) {
         // "form": the Bluestein form that runs ("" for an axis without one);
         // "fused": the length-M form of this padded length (0 five passes, 1
         // two, 2 one), which does not run where "half_q" > 0, the length of the
-        // one-pass form's transforms
+        // one-pass form's transforms; "mixed_lanes": mixed-radix transforms per
+        // thread (2: the kernel over pairs), "mixed_w" per CTA
         auto axis = [](const gb300fft::AnyAxis &ax, char *o, int cap) {
             const int fused = ax.half ? (ax.M > 8192 ? 0 : ax.M > 2048 ? 1 : 2) : ax.fused ? (ax.fused_one ? 2 : 1) : 0;
             const char *form = !ax.M ? "" : ax.half ? "half" : fused == 2 ? "one_pass" : fused == 1 ? "two_pass" : "five_pass";
             snprintf(o, cap,
                      "{\"n\": %d, \"bluestein_m\": %d, \"form\": \"%s\", \"fused\": %d, \"half_q\": %d, \"mixed\": %d, "
-                     "\"mixed_fourstep\": [%d, %d]}",
-                     ax.n, ax.M, form, fused, ax.half ? ax.half->q : 0, ax.mixed ? 1 : 0, ax.n1, ax.n2);
+                     "\"mixed_lanes\": %d, \"mixed_w\": %d, \"mixed_fourstep\": [%d, %d]}",
+                     ax.n, ax.M, form, fused, ax.half ? ax.half->q : 0, ax.mixed ? 1 : 0,
+                     !ax.mixed ? 0 : ax.ml.rmax > 0 ? 2 : 1, ax.mixed ? ax.ml.W : 0, ax.n1, ax.n2);
         };
         char x[256], y[256];
         axis(ap.x, x, sizeof x);
