@@ -350,8 +350,8 @@ struct MixedLaunch {
 // The kernels (fft_mixed_pair.cuh), compiled per largest radix: threads whose
 // registers fill an SM (96 and 128 each).
 constexpr int mixed_pair_threads(int rmax) { return rmax <= 13 ? 640 : 512; }
-const void *mixed_pair13_fn(bool cols, bool fs);
-const void *mixed_pair16_fn(bool cols, bool fs);
+const void *mixed_pair13_fn(bool cols);
+const void *mixed_pair16_fn(bool cols);
 constexpr int kMixedOneThreads = 1024;  // of 64 registers
 const void *mixed_one_fn(bool cols, bool fs);
 bool mixed_factor(int n, MixedStages *st);  // false unless n = 2^a 3^b 5^c 7^d 11^e 13^f <= kMixedMaxN

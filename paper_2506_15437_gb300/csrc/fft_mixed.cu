@@ -53,7 +53,9 @@ __global__ void k_mixed_twiddles(float2 *t, int Ns, int R) {
 }
 
 const void *mixed_fn(int rmax, bool cols, bool fs) {
-    return rmax == 0 ? mixed_one_fn(cols, fs) : rmax <= 13 ? mixed_pair13_fn(cols, fs) : mixed_pair16_fn(cols, fs);
+    if (rmax == 0) return mixed_one_fn(cols, fs);
+    if (fs) return nullptr;  // no four-step kernel over pairs
+    return rmax <= 13 ? mixed_pair13_fn(cols) : mixed_pair16_fn(cols);
 }
 int mixed_threads(int rmax) { return rmax == 0 ? kMixedOneThreads : mixed_pair_threads(rmax); }
 
@@ -63,7 +65,7 @@ int mixed_threads(int rmax) { return rmax == 0 ? kMixedOneThreads : mixed_pair_t
 // plan-sized limit would let a plan created later (or concurrently, on
 // another thread) lower it below what an earlier plan launches with.
 bool smem_ok(const void *fn, size_t smem) {
-    if (smem > kMixedMaxSmem) return false;
+    if (!fn || smem > kMixedMaxSmem) return false;
     if (smem > 48 * 1024 &&
         cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMixedMaxSmem) != cudaSuccess)
         return false;

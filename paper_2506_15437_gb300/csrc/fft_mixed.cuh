@@ -200,10 +200,6 @@ __device__ __forceinline__ int fdiv(int x, int d, uint32_t m) {
 // to even, so each butterfly's twiddles are whole 16-byte pairs.
 __host__ __device__ constexpr int mixed_tw_stride(int R) { return (R - 1 + 1) & ~1; }
 
-// padded shared-memory index: one spare slot after every 2^ps elements
-// (ps = 31: no padding, since every index is below 2^31)
-__device__ __forceinline__ int padx(int x, int ps) { return x + (x >> ps); }
-
 // w_n^e from the two factor tables, w_n^e = hi[e >> L] lo[e & (2^L - 1)]
 __device__ __forceinline__ float2 fs_root(const FourStepB &fs, int e) {
     return cmul(__ldg(fs.hi + (e >> fs.lshift)), __ldg(fs.lo + (e & fs.lmask)));

@@ -22,7 +22,8 @@
 //
 // Kernels are compiled per largest radix RMAX, since the widest butterfly sets
 // every thread's registers and with them the threads an SM holds.  For launches
-// too small to fill the GPU there is one transform per element instead (V =
+// too small to fill the GPU, for the passes of a four-step transform and for
+// columns of an odd row length there is one transform per element instead (V =
 // float2): twice the threads, half as long a chain of instructions each.
 #pragma once
 
@@ -38,8 +39,7 @@ using namespace mixed;
 
 struct PairGeom {
     int W;        // elements per position (a power of two in the column layout and in four-step rows)
-    int nv;       // valid transforms in this CTA
-    int vec;      // pairs aligned in global memory: 16-byte accesses
+    int nv;       // valid transforms in this CTA (even for pairs of columns)
     int estride;  // element stride within a transform (1 for rows, nx for columns)
     int tstride;  // offset between the CTA's transforms (n for rows, 1 for columns)
     int cstride;  // rows: buffer elements from one transform (pair) to the next
@@ -56,9 +56,10 @@ template <class V, int R, bool COLS, bool FIRST, bool LAST, bool FS>
 __device__ __forceinline__ void pair_stage(const PairGeom &g, const MixedStages &st, int s, V *buf, const float2 *gin,
                                            float2 *gout, const float2 *__restrict__ tw, float si,
                                            const FourStepB &fs) {
-    constexpr bool PAIR = sizeof(V) == sizeof(C2), CFAST = COLS || (LAST && FS), ADJ = PAIR && (COLS || FS);
+    constexpr bool PAIR = sizeof(V) == sizeof(C2), CFAST = COLS || (LAST && FS), ADJ = PAIR && COLS;
+    static_assert(!(PAIR && FS), "four-step passes run one transform per thread");
     const int nb = st.nb[s], Q = st.ns[s], skew = st.skew;
-    const int total = (CFAST ? g.W : ADJ ? (g.nv + 1) >> 1 : g.nv < g.W ? g.nv : g.W) * nb;
+    const int total = (CFAST ? g.W : g.nv < g.W ? g.nv : g.W) * nb;
     for (int idx = threadIdx.x; idx < total; idx += blockDim.x) {
         int c, j;
         if (CFAST) {
@@ -70,8 +71,8 @@ __device__ __forceinline__ void pair_stage(const PairGeom &g, const MixedStages 
         }
         const int t0 = ADJ ? 2 * c : c;                 // lane a's transform
         if (CFAST && t0 >= g.nv) continue;              // past the last column (row)
-        const int tb = ADJ ? g.tstride : g.W * g.tstride;  // lane b's, from lane a's
-        const bool two = t0 + (ADJ ? 1 : g.W) < g.nv;      // lane b holds a transform
+        const int tb = g.W * g.tstride;    // rows: lane b's, from lane a's
+        const bool two = t0 + g.W < g.nv;  // rows: lane b holds a transform
         // butterfly (p, q) and its place in the buffer
         int q = j, pos = FIRST ? j : 0;
         if constexpr (FIRST) {
@@ -102,7 +103,8 @@ __device__ __forceinline__ void pair_stage(const PairGeom &g, const MixedStages 
 #pragma unroll
                 for (int r = 0; r < R; ++r) v[r].y *= si;
             } else {
-                if (COLS && g.vec) {
+                if constexpr (COLS) {
+                    // a pair is 16 bytes: nx and the first column are even
 #pragma unroll
                     for (int r = 0; r < R; ++r) {
                         const float4 u = *reinterpret_cast<const float4 *>(x + r * xs);
@@ -117,25 +119,14 @@ __device__ __forceinline__ void pair_stage(const PairGeom &g, const MixedStages 
                 for (int r = 0; r < R; ++r) v[r].im = mul2(v[r].im, both(si));
             }
             if constexpr (FS) {
-                // element i2 = j + r nb of row m = k1 + t0 (+ 1) times
-                // w_n^{i2 m} = w_n^{j m} w_n^{r nb m}: one gather per thread
-                // and row, the second factor a broadcast along the row
+                // element i2 = j + r nb of row m = k1 + t0 times w_n^{i2 m} =
+                // w_n^{j m} w_n^{r nb m}: one gather per thread, the second
+                // factor a broadcast along the row
                 const int m = fs.k1 + t0;
                 const float2 wa = fs_root(fs, j * m);
-                if constexpr (PAIR) {
-                    const float2 wb = fs_root(fs, two ? j * (m + 1) : 0);
-                    v[0] = cmul(v[0], wa, wb);
+                v[0] = cmul(v[0], wa);
 #pragma unroll
-                    for (int r = 1; r < R; ++r) {
-                        const C2 w =
-                            cmul(lanes(fs_root(fs, r * nb * m), fs_root(fs, two ? r * nb * (m + 1) : 0)), wa, wb);
-                        v[r] = cmul(v[r], lane_a(w), lane_b(w));
-                    }
-                } else {
-                    v[0] = cmul(v[0], wa);
-#pragma unroll
-                    for (int r = 1; r < R; ++r) v[r] = cmul(v[r], cmul(wa, fs_root(fs, r * nb * m)));
-                }
+                for (int r = 1; r < R; ++r) v[r] = cmul(v[r], cmul(wa, fs_root(fs, r * nb * m)));
             }
         } else {
 #pragma unroll
@@ -163,18 +154,17 @@ __device__ __forceinline__ void pair_stage(const PairGeom &g, const MixedStages 
             } else {
 #pragma unroll
                 for (int r = 0; r < R; ++r) v[r].im = mul2(v[r].im, both(si));
-                if (ADJ && g.vec) {
+                if constexpr (COLS) {
 #pragma unroll
                     for (int r = 0; r < R; ++r)
                         *reinterpret_cast<float4 *>(y + r * ys) =
                             make_float4(v[r].re.x, v[r].im.x, v[r].re.y, v[r].im.y);
                 } else {
-                    const int ts = FS ? 1 : tb;
 #pragma unroll
                     for (int r = 0; r < R; ++r) y[r * ys] = lane_a(v[r]);
                     if (two) {
 #pragma unroll
-                        for (int r = 0; r < R; ++r) y[r * ys + ts] = lane_b(v[r]);
+                        for (int r = 0; r < R; ++r) y[r * ys + tb] = lane_b(v[r]);
                     }
                 }
             }
@@ -231,7 +221,6 @@ __global__ void __launch_bounds__(sizeof(V) == sizeof(C2) ? mixed_pair_threads(R
         base = b * (long long)nx * st.n + x0;
         g.estride = nx;
         g.tstride = 1;
-        g.vec = (nx & 1) == 0;
     } else {
         if (FS) {
             // rows k1 .. of transform b; its last group may be narrower
@@ -246,7 +235,6 @@ __global__ void __launch_bounds__(sizeof(V) == sizeof(C2) ? mixed_pair_threads(R
         base = t0 * st.n;
         g.estride = 1;
         g.tstride = st.n;
-        g.vec = FS && (fs.n1 & 1) == 0;
     }
     const float2 *gin = in + base;
     float2 *gout = FS ? out + (base - (long long)fs.k1 * st.n) + fs.k1 : out + base;
@@ -278,10 +266,8 @@ __global__ void __launch_bounds__(sizeof(V) == sizeof(C2) ? mixed_pair_threads(R
 }
 
 template <class V, int RMAX>
-const void *pair_fn(bool cols, bool fs) {
-    return cols ? (const void *)k_mixed_pair<V, RMAX, true, false>
-                : fs ? (const void *)k_mixed_pair<V, RMAX, false, true>
-                     : (const void *)k_mixed_pair<V, RMAX, false, false>;
+const void *pair_fn(bool cols) {
+    return cols ? (const void *)k_mixed_pair<V, RMAX, true, false> : (const void *)k_mixed_pair<V, RMAX, false, false>;
 }
 
 }  // namespace

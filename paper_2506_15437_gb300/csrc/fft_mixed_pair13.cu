@@ -2,5 +2,5 @@
 #include "fft_mixed_pair.cuh"
 
 namespace gb300fft {
-const void *mixed_pair13_fn(bool cols, bool fs) { return pair_fn<C2, 13>(cols, fs); }
+const void *mixed_pair13_fn(bool cols) { return pair_fn<C2, 13>(cols); }
 }  // namespace gb300fft

@@ -2,5 +2,5 @@
 #include "fft_mixed_pair.cuh"
 
 namespace gb300fft {
-const void *mixed_pair16_fn(bool cols, bool fs) { return pair_fn<C2, 16>(cols, fs); }
+const void *mixed_pair16_fn(bool cols) { return pair_fn<C2, 16>(cols); }
 }  // namespace gb300fft
