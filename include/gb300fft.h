@@ -374,6 +374,15 @@ int fft_plan_describe(fft_plan_t p, char *buf, int len);
  * `radices` (capacity 16) or a negative error. */
 int fft_debug_radices(int n, int axis, int *radices);
 
+/* The column pass a plan of power-of-two sizes takes for columns of n points
+ * (2 <= n <= 8192) in `batch` slices of nx columns on a GPU of num_sms SMs: into
+ * the host array info[6] the elements per thread, the tile width, the number of
+ * other elements per thread compiled for that tile, which fft_plan_autotune
+ * times beside it, and these (zeros behind them).  FFT_ERR_INVALID_SIZE for
+ * another n or an nx that is no power of two from 2, FFT_ERR_INVALID_ARG for a
+ * NULL info or a count below 1.  Host only: no device call. */
+int fft_debug_col_choice(int n, int nx, int batch, int num_sms, int *info);
+
 /* The mixed-radix factorisation of length n (2 <= n <= 2^24; Sections 6-7's
  * uneven sizes): for n = 2^a 3^b 5^c 7^d 11^e 13^f <= 14336 one with the fewest
  * stages the compiled radices allow, written to `radices` (capacity 16) and

@@ -58,6 +58,7 @@ SIGNATURES = [
     ("fft_plan_autotune", _I, [_P, _P]),
     ("fft_debug_reorder_map", _I, [_I, _I, _P, _P]),
     ("fft_debug_radices", _I, [_I, _I, ctypes.POINTER(_I)]),
+    ("fft_debug_col_choice", _I, [_I, _I, _I, _I, ctypes.POINTER(_I)]),
     ("fft_debug_row_variant", _I, [_I, _I, _I, ctypes.POINTER(_I)]),
     ("fft_debug_tc_layout", _I, [_I, _I, ctypes.POINTER(ctypes.c_longlong)]),
     ("fft_debug_mixed_plan", _I, [_I, ctypes.POINTER(_I), ctypes.POINTER(_I), ctypes.POINTER(_I)]),

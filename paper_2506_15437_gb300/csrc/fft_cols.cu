@@ -443,6 +443,30 @@ int default_col_w(int n, int nx) {
     return w;
 }
 
+// Elements per thread and tile width (*w) of a column pass over `columns`
+// columns in all, in slices of nx.  Small arrays: narrower tiles (down to
+// 32-byte tile rows) until there is a tile per SM (1024^2: 0.0144 -> 0.0120 ms;
+// 512^2: 0.0105 -> 0.0084).  Still too few tiles to fill the SMs: the latency of
+// one tile counts, and E = 16 has more threads on it (2048 x 512: 0.0146 ->
+// 0.0130 ms).
+int choose_col(int n, int nx, long long columns, int num_sms, int *w) {
+    *w = default_col_w(n, nx);
+    while (*w > 4 && columns / *w < num_sms && col_variant(ilog2(n), preferred_col_e(n, *w / 2), *w / 2)) *w /= 2;
+    return columns / *w < num_sms && n < 4096 ? default_col_e(n) : preferred_col_e(n, *w);
+}
+
+// The other elements per thread compiled for that tile, for the autotuner to
+// time beside choose_col's: into e[3], their count returned.
+int other_col_es(int n, int nx, long long columns, int num_sms, int *e) {
+    int w = 0, count = 0;
+    const int chosen = choose_col(n, nx, columns, num_sms, &w);
+    for (int ce : {16, 32, 64}) {
+        const ColVariant *v = col_variant(ilog2(n), ce, w);
+        if (v && v->e == ce && ce != chosen) e[count++] = ce;
+    }
+    return count;
+}
+
 // Tiles ahead that the column pass asks L2 for, `per_cta` tiles to a CTA:
 // 128-point columns finish a tile sooner than the next one lands (1024 x 128^2,
 // 18 tiles to a CTA: 0.055 -> 0.045 ms); with few tiles to a CTA the first

@@ -45,6 +45,8 @@ bool row_variant_info(int n, int e, int split, int *threads, int *rows_per_cta, 
 int default_col_e(int n);
 int preferred_col_e(int n, int w);
 int default_col_w(int n, int nx);
+int choose_col(int n, int nx, long long columns, int num_sms, int *w);
+int other_col_es(int n, int nx, long long columns, int num_sms, int *e);
 int default_col_pf(int n, long long per_cta);
 
 // Stage radices of the (n, e) schedule, first stage first; returns count.

@@ -337,13 +337,8 @@ int setup_col_axis(fft_plan_s *p, AxisPlan &ax, int n, int nx, long long tiles_p
             return ax.col ? FFT_OK : FFT_ERR_UNSUPPORTED;
         }
     }
-    int w = default_col_w(n, nx);
-    // small arrays: narrower tiles (down to 32-byte tile rows) until there is
-    // a tile per SM (1024^2: 0.0144 -> 0.0120 ms; 512^2: 0.0105 -> 0.0084)
-    while (w > 4 && tiles_per_w / w < p->num_sms && col_variant(ilog2(n), preferred_col_e(n, w / 2), w / 2)) w /= 2;
-    // still too few tiles to fill the SMs: the latency of one tile counts, and
-    // E = 16 has more threads on it (2048 x 512: 0.0146 -> 0.0130 ms)
-    int e = tiles_per_w / w < p->num_sms && n < 4096 ? default_col_e(n) : preferred_col_e(n, w);
+    int w = 0;
+    int e = choose_col(n, nx, tiles_per_w, p->num_sms, &w);
     if (sc.col_kind == kColTile && sc.col_e > 0 && col_variant(ilog2(n), sc.col_e, w)) e = sc.col_e;
     if (sc.col_kind == kColTile && sc.col_w >= 2 && sc.col_w <= nx && col_variant(ilog2(n), e, sc.col_w)) w = sc.col_w;
     ax.col = col_variant(ilog2(n), e, w);
@@ -1472,11 +1467,11 @@ int fft_plan_autotune(fft_plan_t p, void *stream) {
                         cands.push_back(f);
                     }
                 }
-                for (int ce : {16, 64}) {
-                    if (!col_variant(ilog2(cn), ce, default_col_w(cn, p->nx)) || ce == preferred_col_e(cn, default_col_w(cn, p->nx)))
-                        continue;
+                int others[3];
+                const int count = other_col_es(cn, p->nx, (long long)p->nx * p->batch * split, p->num_sms, others);
+                for (int k = 0; k < count; ++k) {
                     Schedule d = c;
-                    d.col_e = ce;
+                    d.col_e = others[k];
                     cands.push_back(d);
                 }
                 if (cluster_cols_width(cn, 16, 2, p->nx) > 0) {
@@ -1634,6 +1629,15 @@ int fft_debug_radices(int n, int axis, int *radices) {
     if (!is_pow2(n) || n > 8192 || !radices || (axis != 0 && axis != 1)) return FFT_ERR_INVALID_ARG;
     const int e = axis == 0 ? default_row_e(n) : default_col_e(n);
     return schedule_radices(n, e, radices);
+}
+
+int fft_debug_col_choice(int n, int nx, int batch, int num_sms, int *info) {
+    if (!info || batch < 1 || num_sms < 1) return FFT_ERR_INVALID_ARG;
+    if (!is_pow2(n) || n < 2 || n > 8192 || !is_pow2(nx) || nx < 2) return FFT_ERR_INVALID_SIZE;
+    info[0] = gb300fft::choose_col(n, nx, (long long)nx * batch, num_sms, &info[1]);
+    info[2] = gb300fft::other_col_es(n, nx, (long long)nx * batch, num_sms, info + 3);
+    for (int k = info[2]; k < 3; ++k) info[3 + k] = 0;
+    return FFT_OK;
 }
 
 int fft_debug_tc_layout(int n, int kind, long long *info) {
