@@ -216,21 +216,29 @@ void tune_cache_store(int nx, int ny, int batch, int prec, const Schedule &sc, f
     fclose(f);
 }
 
+// Elements per thread of the FP32 row pass.  512- and 1024-point rows: E = 32
+// makes them two stages with one exchange (2^24 points: 0.0433 -> 0.0422 ms and
+// 0.0440 -> 0.0430; 2^21 points of 1024 0.0080 -> 0.0068), where there are rows
+// enough for its fewer threads.  4096-point rows have three stages either way;
+// their 128-thread CTAs win once there are rows for several rounds of them (2^25
+// points 0.0957 -> 0.0945 ms, 2^26 0.184 -> 0.181; 2^22 points 0.0136 -> 0.0145,
+// so not there).  Not where something asks for E = 16: the column pre-split's
+// kernels, the one-launch small transforms and the landing ring, where it is
+// switched on.
+int choose_row_e(const fft_plan_s *p, int n, const Schedule &sc) {
+    const long long points = (long long)p->nx * p->ny * p->batch;
+    const bool wide = n == 512 || n == 1024 ? points >= 1 << 20 : n == 4096 && points >= 1 << 24;
+    const bool twod = p->nx > 1 && p->ny > 1;
+    if (!wide || (sc.ring && ring_rows_available(n)) ||
+        (twod && (sc.split == 2 || small2d_available(p->nx, p->ny, p->batch, 16))))
+        return default_row_e(n);
+    return 32;
+}
+
 int setup_row_axis(fft_plan_s *p, AxisPlan &ax, int n, const Schedule &sc) {
     ax.n = n;
     if (n == 1) return FFT_OK;
-    int e = default_row_e(n);
-    // 512- and 1024-point rows: E = 32 makes them two stages with one exchange
-    // (2^24 points: 0.0433 -> 0.0422 ms and 0.0440 -> 0.0430; 2^21 points of 1024
-    // 0.0080 -> 0.0068), where there are rows enough for its fewer threads and
-    // nothing asks for E = 16 (the column pre-split's kernels and the one-launch
-    // small transforms).  4096-point rows have three stages either way; their
-    // 128-thread CTAs win once there are rows for several rounds of them (2^25
-    // points 0.0957 -> 0.0945 ms, 2^26 0.184 -> 0.181; 2^22 points 0.0136 ->
-    // 0.0145, so not there).
-    if ((long long)p->nx * p->ny * p->batch >= (n == 4096 ? 1 << 24 : 1 << 20) && (n == 512 || n == 1024 || n == 4096) &&
-        !(p->nx > 1 && p->ny > 1 && (sc.split == 2 || small2d_available(p->nx, p->ny, p->batch, 16))))
-        e = 32;
+    int e = choose_row_e(p, n, sc);
     if (p->prec == FFT_PREC_SPLIT_FP16_TC) {
         if (!tc_rows_available(n)) return FFT_ERR_UNSUPPORTED;
         e = 16;
