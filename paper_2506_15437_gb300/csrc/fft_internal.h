@@ -240,6 +240,8 @@ struct AxisPlan {
     const RowVariant *row = nullptr;
     const ColVariant *col = nullptr;
     float2 *tw = nullptr;
+    const RowVariant *weighted_row = nullptr;  // rows under a weight array, where another kernel is the faster one
+    float2 *weighted_tw = nullptr;
     int n = 1;
     int grid = 0;  // column pass: persistent grid size
     int pf = 0;    // column pass: L2 prefetch distance in tiles

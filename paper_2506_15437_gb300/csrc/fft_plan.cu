@@ -257,6 +257,17 @@ int setup_row_axis(fft_plan_s *p, AxisPlan &ax, int n, const Schedule &sc) {
         if (!ax.tw) return FFT_ERR_ALLOC;
         if (build_twiddles(ax.tw, n, ax.row->e, 0) != cudaSuccess) return FFT_ERR_CUDA;
     }
+    // 4096-point rows under a weight array keep 16 elements per thread: with the
+    // weights a thread of 32 waits longer for its loads than the fewer threads
+    // gain (weighted adjoint of 2^24, 2^25 and 2^26 points 0.124, 0.233 and 0.440
+    // ms against 0.128, 0.241 and 0.455; under a scale alone 32 is the faster,
+    // 0.193 against 0.198; at 512 and 1024 points both ways, 0.104 against 0.107)
+    if (n == 4096 && ax.row->e == 32 && sc.row_e <= 0 && p->prec == FFT_PREC_FP32) {
+        ax.weighted_row = row_variant(ilog2(n), 16);
+        ax.weighted_tw = dev_alloc<float2>(p, ax.weighted_row->tw_size);
+        if (!ax.weighted_tw) return FFT_ERR_ALLOC;
+        if (build_twiddles(ax.weighted_tw, n, 16, 0) != cudaSuccess) return FFT_ERR_CUDA;
+    }
     if (ax.row->smem > 48 * 1024)
         cudaFuncSetAttribute(ax.row->fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ax.row->smem);
     p->row_persist = sc.row_persist;
@@ -1007,10 +1018,13 @@ int run_dense(fft_plan_s *p, const void *in, void *out, int sign, const float *w
     const bool stream =
         planar || (two_pass && src != dst && cp.stream && !p->ring && cp.cl_c == 0 && cp.pair_e == 0);
     float2 *row_dst = planar ? p->planar_work : dst;
+    const bool own = weight && p->rows.weighted_row;  // P == 1: E = 32 has no pre-split at 4096 points
+    const RowVariant &rv = own ? *p->rows.weighted_row : *p->rows.row;
+    const float2 *rtw = own ? p->rows.weighted_tw : p->rows.tw;
     int &grid = p->row_grid[weight ? 1 : 0][P > 1 ? 1 : 0];
     if (grid == 0)
         grid = p->ring ? ring_rows_grid(p->rows.n, nrows, P, p->num_sms, weight != nullptr)
-                       : row_grid(*p->rows.row, nrows, p->num_sms, weight != nullptr, P,
+                       : row_grid(rv, nrows, p->num_sms, weight != nullptr, P,
                                   p->row_persist < 0 ? P > 1 : p->row_persist != 0);
     if (p->ev[0] && pass_event(p, 0, s) != cudaSuccess) return FFT_ERR_CUDA;
     const bool land = P == 2 && !weight && !p->ring && p->sched.row_land &&
@@ -1021,7 +1035,7 @@ int run_dense(fft_plan_s *p, const void *in, void *out, int sign, const float *w
                                 p->num_sms, p->sched.land_pf, s)
         : p->ring ? launch_rows_ring(p->rows.n, src, dst, p->rows.tw, p->twp, nrows, p->ny, P, inv ? 1 : 0,
                                    (inv && !two_pass) ? 1 : 0, weight, wscale, wscale_dev, p->status, grid, s)
-                : launch_rows(*p->rows.row, src, row_dst, p->rows.tw, p->twp, nrows, p->ny, P, inv ? 1 : 0,
+                : launch_rows(rv, src, row_dst, rtw, p->twp, nrows, p->ny, P, inv ? 1 : 0,
                               (inv && !two_pass) ? 1 : 0, weight, wscale, wscale_dev, grid, p->row_pf,
                               stream ? cp.perm_t : 0,
                               stream ? cp.perm_g : 0, planar ? 1 : 0, s);
@@ -1612,11 +1626,11 @@ int fft_plan_describe(fft_plan_t p, char *buf, int len) {
         }
         k = snprintf(tmp, sizeof tmp,
                      "{\"kind\": \"dense\", \"precision\": \"%s\", \"rows\": {\"kernel\": \"%s<%d,%d,split%d>\", "
-                     "\"n\": %d, \"e\": %d, \"radices\": %s, \"persistent\": %d}, "
+                     "\"n\": %d, \"e\": %d, \"weighted_e\": %d, \"radices\": %s, \"persistent\": %d}, "
                      "\"cols\": {\"kernel\": \"%s<%d,%d,%d>\", \"n\": %d, \"e\": %d, \"w\": %d, \"radices\": %s, "
                      "\"grid\": %d}, \"split\": %d, \"col_tma_store\": %d, \"one_launch\": %d}",
                      tc ? "split_fp16_tc" : "fp32", tc ? (p->rows.tc32 ? (tc32_land_used(p, (long long)p->nx * p->ny * p->batch / p->rows.n, p->split) ? "k_rows_tc32_land" : "k_rows_tc32") : p->tcg ? "k_rows_tcgen05" : "k_rows_mmasync") : (p->ring ? "k_rows_ring" : (p->split == 2 && p->sched.row_land && p->rows.row && land_rows_available(p->rows.n, p->rows.row->e)) ? "k_rows_land" : "k_rows"), p->rows.n, re,
-                     p->split, p->rows.n, re, r1, p->row_persist < 0 ? (p->split > 1) : p->row_persist,
+                     p->split, p->rows.n, re, p->rows.weighted_row ? p->rows.weighted_row->e : re, r1, p->row_persist < 0 ? (p->split > 1) : p->row_persist,
                      !cp.col ? "none" : tc ? (tcs ? "k_cols_tc_stream" : cp.tc32 ? "k_cols_tc32" : cp.tcg ? "k_cols_tcgen05" : "k_cols_mmasync") : (cp.cl_c > 0 ? "k_cols_cluster" : cp.pair_e > 0 ? "k_cols_pair" : (cp.stream && !p->ring) ? "k_cols_stream" : "k_cols"), cp.n,
                      cp.cl_c > 0 ? cp.cl_e : cp.pair_e > 0 ? cp.pair_e : cp.col ? (tc ? (tcs ? 64 : cp.tc32 ? 32 : 16) : cp.col->e) : 0,
                      cp.cl_c > 0 ? cp.cl_c : cp.pair_e > 0 ? pair_cols_width(cp.n, cp.pair_e, p->nx) : cp.col ? (tc ? cp.tc_w : cp.col->w) : 0,
