@@ -162,20 +162,33 @@ __device__ __forceinline__ float2 lane_a(C2 v) { return make_float2(v.re.x, v.im
 __device__ __forceinline__ float2 lane_b(C2 v) { return make_float2(v.re.y, v.im.y); }
 __device__ __forceinline__ C2 lanes(float2 a, float2 b) { return {make_float2(a.x, b.x), make_float2(a.y, b.y)}; }
 
-// (u - v) * exp(-2*pi*i*q/64), 0 <= q < 32 a constant after unrolling
-__device__ __forceinline__ float2 sub_root64(float2 u, float2 v, int q) { return mul_root64(csub(u, v), q); }
-__device__ __forceinline__ C2 sub_root64(C2 u, C2 v, int q) {
-    if (q == 16) return {sub2(u.im, v.im), sub2(v.re, u.re)};  // times -i: no negation left over
-    const C2 d = csub(u, v);
+// d * exp(-2*pi*i*q/64), 0 <= q < 48 a constant after unrolling, no multiple of 16
+// but 0
+__device__ __forceinline__ C2 mul_root64(C2 d, int q) {
     if (q == 0) return d;
-    if (q == 8 || q == 24) {
+    if ((q & 15) == 8) {
         const float h = 0.7071067811865475f;
         const float2 sum = add2(d.re, d.im), dif = sub2(d.im, d.re);
-        return q == 8 ? C2{mul2(sum, both(h)), mul2(dif, both(h))} : C2{mul2(dif, both(h)), mul2(sum, both(-h))};
+        return q == 8    ? C2{mul2(sum, both(h)), mul2(dif, both(h))}
+               : q == 24 ? C2{mul2(dif, both(h)), mul2(sum, both(-h))}
+                         : C2{mul2(sum, both(-h)), mul2(dif, both(-h))};
     }
     const float c = cos64(q), s = sin64(q);
     return {fma2(d.im, both(s), mul2(d.re, both(c))), fma2(d.re, both(-s), mul2(d.im, both(c)))};
 }
+
+// (u - v) * exp(-2*pi*i*q/64), 0 <= q < 32 a constant after unrolling
+__device__ __forceinline__ float2 sub_root64(float2 u, float2 v, int q) { return mul_root64(csub(u, v), q); }
+__device__ __forceinline__ C2 sub_root64(C2 u, C2 v, int q) {
+    if (q == 16) return {sub2(u.im, v.im), sub2(v.re, u.re)};  // times -i: no negation left over
+    return mul_root64(csub(u, v), q);
+}
+
+// a - i b and a + i b
+__device__ __forceinline__ float2 sub_i(float2 a, float2 b) { return make_float2(a.x + b.y, a.y - b.x); }
+__device__ __forceinline__ C2 sub_i(C2 a, C2 b) { return {add2(a.re, b.im), sub2(a.im, b.re)}; }
+__device__ __forceinline__ float2 add_i(float2 a, float2 b) { return make_float2(a.x - b.y, a.y + b.x); }
+__device__ __forceinline__ C2 add_i(C2 a, C2 b) { return {sub2(a.re, b.im), add2(a.im, b.re)}; }
 
 // One radix-2 decimation-in-frequency level of span H over R registers:
 // (u, v) -> (u + v, (u - v) * w_{2H}^k).  Levels recurse at compile time so
@@ -196,6 +209,32 @@ __device__ __forceinline__ void dif_level(V *a) {
     }
 }
 
+// Two such levels as one of radix 4 and span Q: the rotations between the two
+// radix-2 levels fold into those behind the second, so a value is rotated (and
+// rounded) at most once in two levels.  Results lie where the two radix-2 levels
+// leave them.  Q / 4 levels follow; a last odd one is of radix 2.
+template <int R, int Q, class V>
+__device__ __forceinline__ void dif_level4(V *a) {
+    if constexpr (Q >= 1) {
+        constexpr int U = 16 / Q;  // w_{4Q} = w_64^U
+#pragma unroll
+        for (int blk = 0; blk < R; blk += 4 * Q) {
+#pragma unroll
+            for (int k = 0; k < Q; ++k) {
+                V *p = a + blk + k;
+                const V s02 = cadd(p[0], p[2 * Q]), d02 = csub(p[0], p[2 * Q]);
+                const V s13 = cadd(p[Q], p[3 * Q]), d13 = csub(p[Q], p[3 * Q]);
+                p[0] = cadd(s02, s13);
+                p[Q] = sub_root64(s02, s13, 2 * k * U);
+                p[2 * Q] = mul_root64(sub_i(d02, d13), k * U);
+                p[3 * Q] = mul_root64(add_i(d02, d13), 3 * k * U);
+            }
+        }
+        if constexpr (Q >= 4) dif_level4<R, Q / 4>(a);
+        else if constexpr (Q == 2) dif_level<R, 1>(a);
+    }
+}
+
 // a[K] = t[bitrev(K)] for K = 0..R-1, every index a constant expression.
 template <int R, int K, class V>
 __device__ __forceinline__ void bitrev_gather(V *a, const V *t) {
@@ -207,12 +246,20 @@ __device__ __forceinline__ void bitrev_gather(V *a, const V *t) {
 }
 
 // In-register length-R DFT (forward sign), natural order in and out,
-// R a power of two <= 64: radix-2 DIF levels, then a compile-time
-// bit-reversal of register names.
-template <int R, class V>
+// R a power of two <= 64: DIF levels, then a compile-time bit-reversal of
+// register names.  Levels of radix 4 from FOUR points on, of radix 2 below.
+// Every rotation rounds: with radix-2 levels a pass in 32- and 64-point stages,
+// which saves an exchange, came out further from the exact result than one in
+// stages of 16 (relative L2 of Gaussian columns of 1024 points 1.182e-7 against
+// 1.128e-7, 2048 points 1.256e-7 against 1.185e-7); with radix 4 it is the closer
+// one (1.104e-7, 1.167e-7; 4096 points 1.330e-7 -> 1.229e-7).  Fewer operations
+// too: 4 x 2^24 points 0.485 -> 0.470 ms, 8 x 2048^2 loss and gradient 0.414 ->
+// 0.407.
+template <int R, int FOUR = 32, class V>
 __device__ __forceinline__ void dft(V *a) {
     if constexpr (R > 1) {
-        dif_level<R, R / 2>(a);
+        if constexpr (R >= FOUR) dif_level4<R, R / 4>(a);
+        else dif_level<R, R / 2>(a);
         V t[R];
 #pragma unroll
         for (int k = 0; k < R; ++k) t[k] = a[k];
@@ -252,12 +299,14 @@ struct FftPolicy {
     __device__ __forceinline__ void butterfly(T *a) const { dft<R>(a); }
     __device__ __forceinline__ T twiddle(T a, float2 w) const { return cmul(a, w); }
 };
-// two transforms per thread, one per lane of C2
+// two transforms per thread, one per lane of C2; radix-4 levels from 16 points:
+// the half-length Bluestein's outer rotations cost what they save (16384 x 4093:
+// 2.83e-7 with radix 2, 2.67e-7, and 0.553 -> 0.538 ms; the length-M form 2.78e-7)
 struct PairPolicy {
     using T = C2;
     static constexpr bool kUsesTwiddles = true;
     template <int R>
-    __device__ __forceinline__ void butterfly(T *a) const { dft<R>(a); }
+    __device__ __forceinline__ void butterfly(T *a) const { dft<R, 16>(a); }
     __device__ __forceinline__ T twiddle(T a, float2 w) const { return cmul(a, w); }
 };
 struct MovePolicy {

@@ -62,17 +62,13 @@ __host__ __device__ constexpr OddRoots<R> odd_roots() {
 //   y_m     = a_0 + sum_k t_k cos(2 pi k m / R) - i sum_k d_k sin(2 pi k m / R)
 //   y_{R-m} = a_0 + sum_k t_k cos(2 pi k m / R) + i sum_k d_k sin(2 pi k m / R)
 // with t_k = a_k + a_{R-k}, d_k = a_k - a_{R-k}, k, m = 1 .. (R-1)/2.
-// a + c b and a - i b, a + i b, for one transform (float2) or two (C2)
+// a + c b, for one transform (float2) or two (C2)
 __device__ __forceinline__ float2 axpy(float c, float2 b, float2 a) {
     return make_float2(fmaf(c, b.x, a.x), fmaf(c, b.y, a.y));
 }
 __device__ __forceinline__ C2 axpy(float c, C2 b, C2 a) { return {fma2(both(c), b.re, a.re), fma2(both(c), b.im, a.im)}; }
 __device__ __forceinline__ float2 scaled(float c, float2 b) { return make_float2(c * b.x, c * b.y); }
 __device__ __forceinline__ C2 scaled(float c, C2 b) { return {mul2(both(c), b.re), mul2(both(c), b.im)}; }
-__device__ __forceinline__ float2 sub_i(float2 a, float2 b) { return make_float2(a.x + b.y, a.y - b.x); }
-__device__ __forceinline__ C2 sub_i(C2 a, C2 b) { return {add2(a.re, b.im), sub2(a.im, b.re)}; }
-__device__ __forceinline__ float2 add_i(float2 a, float2 b) { return make_float2(a.x - b.y, a.y + b.x); }
-__device__ __forceinline__ C2 add_i(C2 a, C2 b) { return {sub2(a.re, b.im), add2(a.im, b.re)}; }
 
 template <int R, class V>
 __device__ __forceinline__ void dft_odd(V *a) {
