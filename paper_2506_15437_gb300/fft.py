@@ -7,6 +7,7 @@ pointers and the current stream through ctypes.
 from __future__ import annotations
 
 import ctypes
+import functools
 import threading
 
 import torch
@@ -18,11 +19,17 @@ _PREC = {"fp32": N.FFT_PREC_FP32, "split_tc": N.FFT_PREC_SPLIT_FP16_TC,
          "split_fp16_tc": N.FFT_PREC_SPLIT_FP16_TC}
 
 
+_Tensor, _C64 = torch.Tensor, torch.complex64
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)  # none in a torch without CUDA
+_transforms_active, _tracing_state = torch._C._are_functorch_transforms_active, torch._C._get_tracing_state
+_is_compiling = torch.compiler.is_compiling
+
+
 def _stream_handle(device) -> int:
     # the current stream's handle without building a Stream object (0.1 us
     # against 2.0)
     index = torch.device(device).index
-    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device() if index is None else index)
+    return _raw_stream(torch.cuda.current_device() if index is None else index)
 
 
 def _check_tensor(t: torch.Tensor, dtype, name: str):
@@ -40,16 +47,12 @@ def _values(t: torch.Tensor) -> torch.Tensor:
     """t with a lazy conjugation or negation carried out.  The kernels read
     t's memory, which such a view (x.conj(), the gradient that reaches
     fft2(x).conj()) leaves as it was; contiguous() keeps the view."""
-    if t.is_conj():
-        t = t.resolve_conj()
-    if t.is_neg():
-        t = t.resolve_neg()
-    return t
+    return t.resolve_conj().resolve_neg()
 
 
 def _input(t: torch.Tensor, dtype, name: str) -> torch.Tensor:
     _check_tensor(t, dtype, name)
-    return _values(t)
+    return _values(t) if t.is_conj() or t.is_neg() else t
 
 
 def _check_output(t: torch.Tensor, dtype, name: str):
@@ -72,26 +75,31 @@ class Plan:
         if not self._p:
             raise N.FFTError(lib.fft_last_error(), f"fft_plan_create({nx}, {ny}, {batch})")
 
-    @property
+    @functools.cached_property
     def numel(self) -> int:
         return self.nx * self.ny * self.batch
 
     def _io(self, x, out):
-        x = _input(x, torch.complex64, "input")
-        if x.numel() != self.numel:
-            raise ValueError(f"input has {x.numel()} elements, plan expects {self.numel}")
+        # a tensor whose memory is the plan's array as it stands passes on
+        # inline tests (the calls below cost a 5 us transform 0.5 us)
+        numel = self.numel
+        if not (isinstance(x, _Tensor) and x.is_cuda and x.dtype is _C64 and x.is_contiguous()
+                and x.numel() == numel and not x.is_conj() and not x.is_neg()):
+            x = _input(x, _C64, "input")
+            if x.numel() != numel:
+                raise ValueError(f"input has {x.numel()} elements, plan expects {numel}")
         if out is None:
             out = torch.empty_like(x)
-        else:
-            _check_output(out, torch.complex64, "out")
-            if out.numel() != self.numel:
+        elif not (isinstance(out, _Tensor) and out.is_cuda and out.dtype is _C64 and out.is_contiguous()
+                  and out.numel() == numel and not out.is_conj() and not out.is_neg()):
+            _check_output(out, _C64, "out")
+            if out.numel() != numel:
                 raise ValueError("out has the wrong size")
         return x, out
 
     def execute(self, x: torch.Tensor, out: torch.Tensor | None = None) -> torch.Tensor:
         x, out = self._io(x, out)
-        rc = self._lib.fft_execute(self._p, x.data_ptr(), out.data_ptr(),
-                                   torch._C._cuda_getCurrentRawStream(x.get_device()))
+        rc = self._lib.fft_execute(self._p, x.data_ptr(), out.data_ptr(), _raw_stream(x.get_device()))
         if rc:
             N.check(rc, "fft_execute")
         return out
@@ -280,7 +288,8 @@ _cache_lock = threading.Lock()
 
 
 def get_plan(nx: int, ny: int, batch: int, inverse: bool, precision: str, device) -> Plan:
-    key = (nx, ny, batch, inverse, precision, torch.device(device).index)
+    key = (nx, ny, batch, inverse, precision,
+           device.index if type(device) is torch.device else torch.device(device).index)
     p = _cache.get(key)
     if p is not None:
         return p
@@ -296,7 +305,7 @@ def get_plan(nx: int, ny: int, batch: int, inverse: bool, precision: str, device
 def _shape(x: torch.Tensor):
     if x.dim() < 2:
         raise ValueError("fft2 needs at least 2 dimensions ([..., ny, nx])")
-    ny, nx = x.shape[-2], x.shape[-1]
+    ny, nx = x.shape[-2:]
     return nx, ny, max(1, x.numel() // max(1, nx * ny))
 
 
@@ -305,9 +314,9 @@ def _plain(x) -> bool:
     tensor that no gradient is wanted of, outside forward-mode AD, functorch
     transforms, tracing and compilation.  Function.apply costs more than the
     rest of a small call (256 x 256: 24 us a call through it)."""
-    return (type(x) is torch.Tensor and not (x.requires_grad and torch.is_grad_enabled())
-            and not torch._C._are_functorch_transforms_active() and forward_ad._current_level < 0
-            and torch._C._get_tracing_state() is None and not torch.compiler.is_compiling())
+    return (type(x) is _Tensor and not (x.requires_grad and torch.is_grad_enabled())
+            and not _transforms_active() and forward_ad._current_level < 0
+            and _tracing_state() is None and not _is_compiling())
 
 
 class FFT2Function(torch.autograd.Function):
@@ -417,6 +426,8 @@ def reorder_map(n: int, axis: int = 0, device="cuda") -> torch.Tensor:
 
 
 def radices(n: int, axis: int = 0) -> list:
+    """Stage radices of the default schedule (fft_debug_radices); a plan's own
+    are in Plan.describe()."""
     lib = N.load()
     buf = (ctypes.c_int * 16)()
     k = lib.fft_debug_radices(n, axis, buf)

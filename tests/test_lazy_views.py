@@ -53,6 +53,7 @@ def plan(monkeypatch):
 
     monkeypatch.setattr(fft, "_check_tensor", check)
     monkeypatch.setattr(fft, "_stream_handle", lambda device: 0)
+    monkeypatch.setattr(fft, "_raw_stream", lambda index: 0, raising=False)
     monkeypatch.setattr(torch._C, "_cuda_getCurrentRawStream", lambda index: 0, raising=False)
     monkeypatch.setattr(fft, "get_plan", lambda *a: p)
     return p
