@@ -255,21 +255,24 @@ __global__ void __launch_bounds__(ColShape<N, E, W>::THREADS, ColShape<N, E, W>:
             auto keep = [&](int, int, float2 y) { x[m++] = y; };  // X at tt + m * T
             Eng::template run<FftPolicy, true>(v, tile, tw, tt, c, SyncBlock{}, [] {}, keep);
             // w (.) X, its power and the conjugate: X at tt + k * T, k = bb + r *
-            // (E / R0), is the next transform's input (bb, r).  The power is
-            // added up 16 terms at a time, however many a thread holds.
+            // (E / R0), is the next transform's input (bb, r).  A thread of
+            // more than 16 adds its power four terms at a time, so that its
+            // chain of sums is no longer than 16.
             float run = 0.f;
 #pragma unroll
             for (int bb = 0; bb < E / R0; ++bb)
 #pragma unroll
                 for (int r = 0; r < R0; ++r) {
-                    const int k = bb + r * (E / R0);
+                    const int k = bb + r * (E / R0), term = bb * R0 + r;
                     const float wv = __ldg(wt + ((tt + k * T) * nx + c));
-                    run = fmaf(wv, fmaf(x[k].x, x[k].x, x[k].y * x[k].y), run);
-                    v[bb * R0 + r] = make_float2(wv * x[k].x, -(wv * x[k].y));
-                    if ((bb * R0 + r) % 16 == 15) {
-                        part += run;
-                        run = 0.f;
+                    const float power = fmaf(x[k].x, x[k].x, x[k].y * x[k].y);
+                    if constexpr (E <= 16) {
+                        part = fmaf(wv, power, part);
+                    } else {
+                        run = term % 4 == 0 ? wv * power : fmaf(wv, power, run);
+                        if (term % 4 == 3) part += run;
                     }
+                    v[term] = make_float2(wv * x[k].x, -(wv * x[k].y));
                 }
         }
         auto after_reads = [&] {

@@ -1,13 +1,12 @@
-"""The loss partials of the fused column pass (GPU): a thread adds its terms 16
-at a time, however many it holds.
+"""The loss partials of the fused column pass (GPU): a thread's chain of float
+sums is at most 16 long, however many terms it holds (four at a time from 32).
 
 A unit impulse at every slice's origin has the transform 1 everywhere, exactly,
 so a partial is the sum of the weights alone, in the order the kernel adds them.
 The first row block's weights, each thread's first term, are 2^25 and the others
-1: behind 2^25 (ulp 4) a lone 1 is lost, 16 of them added up first are not.  So a
-run of 16 loses 15 of 2^25 and every other run nothing (the sums over threads
-are exact): relative error at most 15 / 2^25.  Runs of 32 and 64 terms lose 31
-and 63.
+1: behind 2^25 (ulp 4) a lone 1 is lost, and a chain of 16 loses 15 of 2^25 (the
+sums over threads are exact): relative error at most 15 / 2^25.  Chains of 32 and
+64 lose 31 and 63.
 """
 import pytest
 
@@ -28,7 +27,7 @@ def g():
 # elements per thread: 16, 32, 32 and, with eight tiles to an SM, 64; 2048 with fewer: 16
 @pytest.mark.parametrize("ny,nx,b,e", [(256, 64, 2, 16), (512, 64, 2, 32), (1024, 64, 2, 32), (2048, 256, 41, 64),
                                        (2048, 64, 2, 16)])
-def test_runs_of_sixteen(g, ny, nx, b, e):
+def test_chains_of_sixteen(g, ny, nx, b, e):
     x = torch.zeros(b, ny, nx, dtype=torch.complex64, device="cuda")
     x[:, 0, 0] = 1
     w = torch.ones(b, ny, nx, device="cuda")
