@@ -23,6 +23,8 @@
 // all tables and constants are for the forward sign only.
 #pragma once
 
+#include <type_traits>
+
 #include <cuda.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -212,9 +214,12 @@ __device__ __forceinline__ void dif_level(V *a) {
 // Two such levels as one of radix 4 and span Q: the rotations between the two
 // radix-2 levels fold into those behind the second, so a value is rotated (and
 // rounded) at most once in two levels.  Results lie where the two radix-2 levels
-// leave them.  Q / 4 levels follow; a last odd one is of radix 2.
+// leave them.  The levels below follow, of radix 4 again; those of 8 points of
+// radix 2 (the same rotations either way, and fewer registers: 512-point rows 110
+// against 116).
 template <int R, int Q, class V>
 __device__ __forceinline__ void dif_level4(V *a) {
+    static_assert(Q == 0 || Q == 1 || Q == 4 || Q == 8 || Q == 16, "16, 32 or 64 points");
     if constexpr (Q >= 1) {
         constexpr int U = 16 / Q;  // w_{4Q} = w_64^U
 #pragma unroll
@@ -230,8 +235,8 @@ __device__ __forceinline__ void dif_level4(V *a) {
                 p[3 * Q] = mul_root64(add_i(d02, d13), 3 * k * U);
             }
         }
-        if constexpr (Q >= 4) dif_level4<R, Q / 4>(a);
-        else if constexpr (Q == 2) dif_level<R, 1>(a);
+        if constexpr (Q == 8) dif_level<R, 4>(a);
+        else dif_level4<R, Q / 4>(a);
     }
 }
 
@@ -292,13 +297,15 @@ struct Sched {
 // path moves integer tags through exactly the same addresses with identity
 // butterflies, which exposes the permutation the data movement realises.
 // ---------------------------------------------------------------------------
-struct FftPolicy {
+template <int FOUR>  // points from which a register DFT has radix-4 levels
+struct FftLevels {
     using T = float2;
     static constexpr bool kUsesTwiddles = true;
     template <int R>
-    __device__ __forceinline__ void butterfly(T *a) const { dft<R>(a); }
+    __device__ __forceinline__ void butterfly(T *a) const { dft<R, FOUR>(a); }
     __device__ __forceinline__ T twiddle(T a, float2 w) const { return cmul(a, w); }
 };
+using FftPolicy = FftLevels<32>;
 // two transforms per thread, one per lane of C2; radix-4 levels from 16 points:
 // the half-length Bluestein's outer rotations cost what they save (16384 x 4093:
 // 2.83e-7 with radix 2, 2.67e-7, and 0.553 -> 0.538 ms; the length-M form 2.78e-7)
@@ -368,7 +375,11 @@ struct Engine {
     __device__ static __forceinline__ void run(typename Pol::T (&v)[E], typename Pol::T *sm,
                                                const float2 *__restrict__ tw, int tt, int c,
                                                Sync sync, AfterReads after_reads, Store store) {
-        run_with<Pol, SRC_IN_SMEM>(Pol{}, v, sm, tw, tt, c, sync, after_reads, store);
+        // 512 = 16 * 32 is as exact with radix-2 levels as 2 * 16 * 16 (1.083e-7
+        // both), and radix 4 costs its kernels registers (512^2 x 64: 92.6 us, with
+        // radix 4 94.4; 2^22 points of rows 11.6 and 12.3)
+        using P = std::conditional_t<N == 512 && std::is_same_v<Pol, FftPolicy>, FftLevels<64>, Pol>;
+        run_with<P, SRC_IN_SMEM>(P{}, v, sm, tw, tt, c, sync, after_reads, store);
     }
 
     // Same, with a policy object (a stateful butterfly, e.g. the tensor-core one).

@@ -7,9 +7,10 @@ every rotation rounds: 1024 points as 32 x 32 came out 5 % further from the exac
 result than as 4 x 16 x 16.  Levels of radix 4 rotate a value at most once in two
 levels.  The bound below is the error of the same lengths in stages of at most
 16 points, emulated in float32 with fused multiply-adds and twiddles rounded once
-(relative L2, Gaussian inputs, 2^19 points; its spread there is 0.1 %); the
-32- and 64-point stages are emulated 1.0 to 3.5 % below it with radix 4 and 0.1 to
-5.6 % above it with radix 2.
+(relative L2, Gaussian inputs, 2^19 points; its spread there is 0.1 %); from 1024
+points the 32- and 64-point stages are emulated 1.0 to 3.5 % below it with radix 4
+and 1.5 to 5.6 % above it with radix 2.  512 = 16 x 32 is on it with radix 2, which
+its kernels keep.
 """
 import numpy as np
 import pytest
