@@ -326,8 +326,9 @@ int fft_plan_status(fft_plan_t p, void *stream);
 /*
  * fft_debug_reorder_map -- the index permutation realised by the kernels'
  * data movement alone.  Runs the row engine (axis 0) or the column engine
- * (axis 1) for length n with every butterfly replaced by the identity and an
- * integer payload, and writes map[i] = the output position of input i.
+ * (axis 1) for length n, in fft_debug_radices' schedule, with every butterfly
+ * replaced by the identity and an integer payload, and writes map[i] = the
+ * output position of input i.
  * With the arithmetic removed, the fused Stockham movement of the kernels is
  * the mixed-radix digit reversal of the stage radices (Section 4's
  * reordering, here folded into the stage loads and stores).  `map` is a
@@ -369,9 +370,11 @@ int fft_plan_autotune(fft_plan_t p, void *stream);
  */
 int fft_plan_describe(fft_plan_t p, char *buf, int len);
 
-/* Stage radices the kernels use for length n along an axis (0 rows, 1
- * columns), first stage first; returns the number of stages written to
- * `radices` (capacity 16) or a negative error. */
+/* Stage radices of the default schedule for length n along an axis (0 rows, 1
+ * columns): stages of at most 16 points, 8192-point rows of at most 32, first
+ * stage first; returns the number of stages written to `radices` (capacity 16)
+ * or a negative error.  Plans with enough rows or tiles take longer stages:
+ * fft_plan_describe has the radices of a plan. */
 int fft_debug_radices(int n, int axis, int *radices);
 
 /* The column pass a plan of power-of-two sizes takes for columns of n points

@@ -13,8 +13,12 @@
 // j^2 mod 2n is reduced in integers and evaluated in FP64 (sincospi), then
 // rounded once to FP32.
 //
-// For M <= 8192 the chirp and filter products are fused into the two
-// transforms (k_blu below): two HBM passes over the padded rows.
+// M = 128 ... 16384 runs as one pass over half-length transforms (k_blu_half
+// below), a shorter M as one pass over length-M transforms with the chirp and
+// filter products fused into them (k_blu), a longer one as five passes.  The
+// length-M forms of 128 <= M <= 8192, one pass or two over the padded rows, and
+// the five passes remain behind GB300FFT_BLUESTEIN_ONEPASS and _FUSED (tests and
+// experiments).
 //
 // A 2D transform whose sizes are not both powers of two runs axis by axis:
 // the x axis over all rows, a tiled transpose, the y axis over the rows of

@@ -257,7 +257,7 @@ __device__ __forceinline__ void bitrev_gather(V *a, const V *t) {
 // which saves an exchange, came out further from the exact result than one in
 // stages of 16 (relative L2 of Gaussian columns of 1024 points 1.182e-7 against
 // 1.128e-7, 2048 points 1.256e-7 against 1.185e-7); with radix 4 it is the closer
-// one (1.104e-7, 1.167e-7; 4096 points 1.330e-7 -> 1.229e-7).  Fewer operations
+// one (1.115e-7, 1.172e-7; 4096 points 1.330e-7 -> 1.229e-7).  Fewer operations
 // too: 4 x 2^24 points 0.485 -> 0.470 ms, 8 x 2048^2 loss and gradient 0.414 ->
 // 0.407.
 template <int R, int FOUR = 32, class V>

@@ -233,7 +233,7 @@ void init_fs_rows() {
 // Elements per thread pass B prefers for row length n: as in the column pass,
 // the fewest that leave one shared-memory exchange (2^24 points, E = 16 against
 // these: 512-point rows 0.068 -> 0.059 ms, 1024 0.080 -> 0.056, 2048 0.080 ->
-// 0.074); 32 at 8192 (two exchanges), 16 otherwise.
+// 0.074); 32 at 8192 (two exchanges), 16 otherwise (and by GB300FFT_FS_EB).
 int fourstep_row_e(int n) { return n == 4096 || n == 2048 ? 64 : n == 8192 || n == 1024 || n == 512 ? 32 : 16; }
 
 // Rows per CTA pass B prefers for row length n: 8 (64-byte store chunks; 256

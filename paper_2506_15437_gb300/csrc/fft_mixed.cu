@@ -181,10 +181,12 @@ void best_factors(int rest, int left, int cap, int *cur, int depth, double sum, 
 }
 
 // Shared-memory wavefronts of the first two warps of every stage, for the
-// radices in this order, `words` pairs per position and each skew 0 .. 7: eight
-// lanes' 16-byte words cost as many wavefronts as the fullest of the eight bank
-// groups holds.  Legs r differ by a constant, which moves every lane's bank
-// alike, so one leg stands for all.
+// radices in this order, `words` elements per position and each skew 0 .. 7:
+// eight lanes' 16-byte pairs cost as many wavefronts as the fullest of the eight
+// bank groups holds.  Legs r differ by a constant, which moves every lane's bank
+// alike, so one leg stands for all.  The one-transform kernels' 8-byte elements
+// are counted as if they were pairs, which ranks orders and skews only
+// approximately (exactly, sixteen lanes would share sixteen banks of 8 bytes).
 void skew_costs(const int *radix, int S, int n, int words, bool cols, bool fs, long long cost[8]) {
     for (int k = 0; k < 8; ++k) cost[k] = 0;
     int Q = n, kdiv = 1;
