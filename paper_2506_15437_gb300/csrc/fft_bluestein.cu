@@ -280,8 +280,8 @@ __global__ void __launch_bounds__(BluShape<N, E>::THREADS, BluShape<N, E>::MINB)
 // exchanges), the FMA pipe (58 %) and, at 16 warps an SM, latency; DRAM moves
 // one read and one write of the signals.  Against the length-M forms this
 // replaces (two passes over padded rows; one pass for M <= 2048; five passes
-// for M = 16384): 16384 x 4093 0.548 / 0.811 ms, 4099 x 4093 0.144 / 0.215, 16627 x 1009
-// 0.130 / 0.205, 32961 x 509 0.121 / 0.192, 4093 x 4099 0.369 / 1.172.  One
+// for M = 16384): 16384 x 4093 0.539 / 0.811 ms, 4099 x 4093 0.141 / 0.215, 16627 x 1009
+// 0.129 / 0.205, 32961 x 509 0.122 / 0.192, 4093 x 4099 0.367 / 1.172.  One
 // thread per half instead of one per pair (scalar butterflies, twice the
 // issue slots, halves added through shared memory): 4099 x 4093 0.186.
 struct SyncHalf {  // barrier over the count >= 32 threads of one row (ids from 1)

@@ -150,7 +150,7 @@ __global__ void __launch_bounds__(ColShape<N, E, W>::THREADS, ColShape<N, E, W>:
 // output and w and writes the adjoint's column half.  Bound by the latency of
 // its exchanges and loads at 8 to 16 warps an SM; writing X back to the tile,
 // sweeping it and loading it again took 16 x 1024^2 (E = 16, with the row pass)
-// 0.182 ms, this 0.141; 64 x 512^2 0.172 -> 0.124, 8 x 2048^2 0.372 -> 0.323,
+// 0.182 ms, this 0.141; 64 x 512^2 0.172 -> 0.124, 8 x 2048^2 0.372 -> 0.319,
 // 256-point columns 0.143 -> 0.124.  The sweep remains at 2048 points with E =
 // 16 (64 registers: X and a three-stage engine spill), the faster form for few
 // tiles.

@@ -17,7 +17,8 @@
 // B as it stores.  Reading the forward result at index (n - k) mod n instead
 // needs no conjugation, but its W-value runs end one element off a sector
 // boundary, so every 32-byte store touches two sectors (4 x 2^24 points:
-// 0.854 ms stored reflected, 0.484 conjugated, the forward 0.482).
+// 0.854 ms stored reflected, 0.484 conjugated, the forward 0.482; since the
+// register DFTs have radix-4 levels 0.470 and 0.477).
 // Two HBM passes, 32 bytes per point, as for the 2D transform.
 //
 // The twiddle of a thread's stage-0 operand e (butterfly b = e / R0, leg

@@ -71,7 +71,7 @@ const ColVariant *wadj_variant(fft_plan_s *p) {
     int w = default_col_w(n, p->nx), e = n == 512 || n == 1024 ? 32 : default_col_e(n);
     if (n == 2048) {
         // 128 KiB tiles with one exchange per transform (E = 64), one to an SM,
-        // where the SMs have eight each or more (8 x 2048^2 0.372 -> 0.323 ms
+        // where the SMs have eight each or more (8 x 2048^2 0.372 -> 0.319 ms
         // against 64 KiB tiles with E = 16); with fewer the last round's idle
         // SMs cost more than that gains (2 x 2048^2 0.104 against 0.110)
         const bool many = p->nx >= 8 && (long long)(p->nx / 8) * p->batch >= 8LL * p->num_sms;
