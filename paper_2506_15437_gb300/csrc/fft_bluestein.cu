@@ -51,6 +51,67 @@ __global__ void k_chirp_filter(float2 *h, const float2 *__restrict__ c, int n, i
     h[m] = idx >= 0 ? make_float2(c[idx].x, -c[idx].y) : make_float2(0.f, 0.f);
 }
 
+// The filter's spectrum in FP64, for padded lengths up to kFilter64M: the filter
+// itself (k_chirp_filter's, unrounded), radix-2 DIF levels in place, and one
+// rounding.  Transformed in FP32, its own error of 0.9 to 1.3e-7 went into every
+// output, and the half-length form came out up to 7 % further from the exact
+// result than the length-M form before it (61 points 1.765e-7, 1009 points
+// 2.389e-7; now 1.487e-7 and 1.918e-7; 4093 points 2.669e-7 -> 2.101e-7).
+__global__ void k_filter64(double2 *h, int n, int M) {
+    const int m = blockIdx.x * blockDim.x + threadIdx.x;
+    if (m >= M) return;
+    const int j = m < n ? m : M - m;
+    double sv = 0.0, cv = 0.0;
+    if (j < n) sincospi((double)((long long)j * j % (2LL * n)) / (double)n, &sv, &cv);
+    h[m] = make_double2(cv, sv);  // conj of the forward chirp
+}
+
+// exp(pi i k / H) = conj(w_{2H}^k)
+__device__ __forceinline__ double2 root64(int k, int H) {
+    double sv, cv;
+    sincospi((double)k / (double)H, &sv, &cv);
+    return make_double2(cv, sv);
+}
+// butterfly k of a block of 2 H elements: (u, v) -> (u + v, (u - v) conj(w))
+__device__ __forceinline__ void dif64(double2 *h, int H, double2 w) {
+    const double2 u = h[0], v = h[H];
+    const double dr = u.x - v.x, di = u.y - v.y;
+    h[0] = make_double2(u.x + v.x, u.y + v.y);
+    h[H] = make_double2(dr * w.x + di * w.y, di * w.x - dr * w.y);
+}
+__global__ void k_dif64(double2 *h, int H, int M) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x, k = i & (H - 1);
+    if (i < M / 2) dif64(h + 2 * (i - k) + k, H, root64(k, H));
+}
+
+// The levels within blocks of C <= kTail64 elements, one to a CTA of C / 2
+// threads, then the spectrum over M, element at0 + e being k bit-reversed: for the
+// forward chirp and, its conjugate (the filter is symmetric), the inverse one.  A
+// plan of 4093 points is created in 0.11 ms with blocks of 512, the roots of all
+// levels tabulated once, in 0.16 with a launch to each level and in 0.18 with
+// blocks of 1024 and no table (an SM's FP64 rate is low); through an FP32 plan
+// 0.12.
+constexpr int kTail64 = 512;
+__global__ void k_dif64_tail(float2 *Hf, float2 *Hi, const double2 *__restrict__ h, int C, int log2M) {
+    __shared__ double2 blk[kTail64], root[kTail64 / 2];
+    const int t = threadIdx.x, at0 = blockIdx.x * C;
+    const double inv = 1.0 / (double)(1 << log2M);
+    for (int e = t; e < C; e += C / 2) blk[e] = h[at0 + e];
+    root[t] = root64(t, C / 2);
+    for (int H = C / 2; H >= 1; H /= 2) {
+        const int k = t & (H - 1);
+        __syncthreads();
+        dif64(blk + 2 * (t - k) + k, H, root[k * (C / 2 / H)]);
+    }
+    __syncthreads();
+    for (int e = t; e < C; e += C / 2) {
+        const unsigned k = __brev((unsigned)(at0 + e)) >> (32 - log2M);
+        const float re = (float)(blk[e].x * inv), im = (float)(blk[e].y * inv);
+        Hf[k] = make_float2(re, im);
+        Hi[k] = make_float2(re, -im);
+    }
+}
+
 __global__ void k_scale(float2 *a, long long count, float s) {
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < count;
          i += (long long)gridDim.x * blockDim.x) {
@@ -514,6 +575,14 @@ cudaError_t build_chirp(float2 *c, int n, int sgn, cudaStream_t s) {
 
 cudaError_t build_chirp_filter(float2 *h, const float2 *c, int n, int M, cudaStream_t s) {
     k_chirp_filter<<<(M + 255) / 256, 256, 0, s>>>(h, c, n, M);
+    return cudaGetLastError();
+}
+
+cudaError_t build_filter_spectra64(float2 *Hf, float2 *Hi, double2 *work, int n, int M, cudaStream_t s) {
+    k_filter64<<<(M + 255) / 256, 256, 0, s>>>(work, n, M);
+    for (int H = M / 2; H >= kTail64; H /= 2) k_dif64<<<(M / 2 + 255) / 256, 256, 0, s>>>(work, H, M);
+    const int C = M < kTail64 ? M : kTail64;
+    k_dif64_tail<<<M / C, C / 2, 0, s>>>(Hf, Hi, work, C, ilog2(M));
     return cudaGetLastError();
 }
 

@@ -308,7 +308,8 @@ struct FftLevels {
 using FftPolicy = FftLevels<32>;
 // two transforms per thread, one per lane of C2; radix-4 levels from 16 points:
 // the half-length Bluestein's outer rotations cost what they save (16384 x 4093:
-// 2.83e-7 with radix 2, 2.67e-7, and 0.553 -> 0.538 ms; the length-M form 2.78e-7)
+// 2.83e-7 with radix 2, 2.67e-7, and 0.553 -> 0.538 ms; the length-M form 2.78e-7;
+// all with the filter's spectrum in FP32)
 struct PairPolicy {
     using T = C2;
     static constexpr bool kUsesTwiddles = true;

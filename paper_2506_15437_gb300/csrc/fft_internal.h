@@ -403,6 +403,11 @@ struct AnyPlan {
 };
 cudaError_t build_chirp(float2 *c, int n, int sgn, cudaStream_t s);
 cudaError_t build_chirp_filter(float2 *h, const float2 *c, int n, int M, cudaStream_t s);
+// the filter spectra of both directions, over M, from a work array of M: the
+// padded lengths of the one- and two-pass forms (longer ones are transformed by a
+// plan, which costs them less time and memory)
+constexpr int kFilter64M = 16384;
+cudaError_t build_filter_spectra64(float2 *Hf, float2 *Hi, double2 *work, int n, int M, cudaStream_t s);
 cudaError_t launch_scale(float2 *a, long long count, float sc, cudaStream_t s);
 cudaError_t launch_blu_pre(const float2 *x, float2 *A, const float2 *c, int n, int M, long long rows, cudaStream_t s);
 cudaError_t launch_blu_mul(float2 *A, const float2 *H, int M, long long rows, cudaStream_t s);

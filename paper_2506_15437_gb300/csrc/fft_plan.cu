@@ -681,17 +681,25 @@ int setup_any_axis(fft_plan_s *p, AnyAxis &ax, int n, long long rows, int cols_n
         ax.H[d] = dev_alloc<float2>(p, ax.M);
         if (!ax.chirp[d] || !ax.H[d]) return FFT_ERR_ALLOC;
     }
-    float2 *filt = dev_alloc<float2>(p, ax.M);
-    if (!filt) return FFT_ERR_ALLOC;
-    // H[d] = F(filter of chirp d) / M through a one-row plan of length M
-    fft_plan_s *one = create_dense(ax.M, 1, 1, FFT_FORWARD, FFT_PREC_FP32, default_schedule(ax.M, 1), &rc);
-    if (!one) return rc;
-    for (int d = 0; d < 2 && rc == FFT_OK; ++d) {
-        if (build_chirp(ax.chirp[d], n, d == 0 ? -1 : 1, 0) != cudaSuccess ||
-            build_chirp_filter(filt, ax.chirp[d], n, ax.M, 0) != cudaSuccess)
-            rc = FFT_ERR_CUDA;
-        if (rc == FFT_OK) rc = run_dense(one, filt, ax.H[d], FFT_FORWARD, nullptr, 1.f, 0);
-        if (rc == FFT_OK && launch_scale(ax.H[d], ax.M, 1.0f / (float)ax.M, 0) != cudaSuccess) rc = FFT_ERR_CUDA;
+    for (int d = 0; d < 2; ++d)
+        if (build_chirp(ax.chirp[d], n, d == 0 ? -1 : 1, 0) != cudaSuccess) return FFT_ERR_CUDA;
+    // H[d] = F(filter of chirp d) / M
+    fft_plan_s *one = nullptr;
+    double2 *work = nullptr;
+    if (ax.M <= kFilter64M) {
+        if (cudaMalloc(&work, ax.M * sizeof(double2)) != cudaSuccess) return FFT_ERR_ALLOC;
+        if (build_filter_spectra64(ax.H[0], ax.H[1], work, n, ax.M, 0) != cudaSuccess) rc = FFT_ERR_CUDA;
+    } else {
+        // through a one-row plan of length M
+        float2 *filt = dev_alloc<float2>(p, ax.M);
+        if (!filt) return FFT_ERR_ALLOC;
+        one = create_dense(ax.M, 1, 1, FFT_FORWARD, FFT_PREC_FP32, default_schedule(ax.M, 1), &rc);
+        if (!one) return rc;
+        for (int d = 0; d < 2 && rc == FFT_OK; ++d) {
+            if (build_chirp_filter(filt, ax.chirp[d], n, ax.M, 0) != cudaSuccess) rc = FFT_ERR_CUDA;
+            if (rc == FFT_OK) rc = run_dense(one, filt, ax.H[d], FFT_FORWARD, nullptr, 1.f, 0);
+            if (rc == FFT_OK && launch_scale(ax.H[d], ax.M, 1.0f / (float)ax.M, 0) != cudaSuccess) rc = FFT_ERR_CUDA;
+        }
     }
     if (rc == FFT_OK && ax.half) {
         const int q = ax.half->q, e = ax.half->e;
@@ -705,7 +713,8 @@ int setup_any_axis(fft_plan_s *p, AnyAxis &ax, int n, long long rows, int cols_n
                  build_blu_half_filter(ax.Hh[1], ax.H[1], q, 0) != cudaSuccess)
             rc = FFT_ERR_CUDA;
     }
-    if (rc == FFT_OK && cudaDeviceSynchronize() != cudaSuccess) rc = FFT_ERR_CUDA;
+    if (cudaDeviceSynchronize() != cudaSuccess && rc == FFT_OK) rc = FFT_ERR_CUDA;
+    cudaFree(work);
     free_plan(one);
     // fused kernels when the padded length is one row pass with the same E
     // (so they share the sub-plan's twiddle table)
